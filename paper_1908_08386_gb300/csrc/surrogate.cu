@@ -3,9 +3,8 @@
 // The forward and adjoint 3x3 convolutions run on the fifth-generation tensor
 // cores (conv_tc.cu: tcgen05.mma with tensor-memory accumulators, TMA-staged
 // operands).  This file holds the rest:
-// weight gradient (wgrad_kernel): one block owns 32 output x 16 input
-//   channels and a strided share of the pixel tiles (split K); its nine warps
-//   take one tap each, so a staged tile serves all taps; products on the
+// weight and bias gradient (wgrad_kernel): one block owns 32 output x 16 input
+//   channels and a strided share of the pixels (split K); products on the
 //   tensor cores by warp-level mma (m16n8k16, BF16, FP32 accumulation) from
 //   operands staged by cp.async and read transposed with ldmatrix (rows of
 //   16 bytes XOR-swizzled so that the eight rows one ldmatrix phase reads fall
@@ -86,113 +85,207 @@ __device__ __forceinline__ int sw64(int r, int c) { return r * 32 + ((c ^ ((r >>
 // ---------------------------------------------------------------------------
 // weight gradient of the 3x3 convolution
 // ---------------------------------------------------------------------------
-constexpr int kTH = 8, kTW = 16;             // pixel tile: 8 rows x 16 pixels
-constexpr int kPH = kTH + 2, kPW = kTW + 2;  // staged input with halo
-constexpr int kWCo = 32, kWCi = 16;  // channels per block
+// A block owns 32 output x 16 input channels of all nine taps and a share of
+// the pieces (8 rows x 16 pixels of one image); each of its eight warps takes
+// pieces of its own and keeps the whole 9 x 32 x 16 accumulator in registers.
+// A row of a piece is one K step of 16 pixels: the output-gradient fragments
+// (two ldmatrix) stay in registers for the three input rows that meet them and
+// the three shifted input fragments of a row serve the three output rows around
+// it, so 36 MMAs follow five ldmatrix (a warp per tap needed three for four).
+// Rows arrive through a five-slot ring per warp filled by cp.async four rows
+// ahead; the warps never wait for one another until the sums are folded.
+// Bound by the warp-level MMA rate and the L2 traffic of re-reading dy for
+// every block of 16 input channels.
+// The bias gradient adds up the same fragments (in FP32): the Cin / 16 blocks
+// that read a piece's dy take turns, one per piece (a kernel of its own walked
+// 1024 pixels per thread).
+// Measured (ncu, 32 maps of 128^2, the network's 14 layers summed): weight and
+// bias gradients 761 + 2450 -> 447 us.
+constexpr int kTH = 8, kTW = 16;       // piece: 8 rows x 16 pixels
+constexpr int kWCo = 32, kWCi = 16;    // channels per block
+constexpr int kWarps = 8;
+constexpr int kItems = kTH + 2;        // input rows of a piece
+constexpr int kSlots = 5;              // kItems % kSlots == 0: slots are compile-time constants
+constexpr int kDRow = kTW * kWCo * 2;  // bytes of a staged dy row: [16 pixels][32 co]
+constexpr int kXRow = 640;             // of an input row: [18 pixels][16 ci], rounded up to 128 bytes
+constexpr int kAcc = 9 * 2 * 2 * 4;    // accumulators per lane
+constexpr int kWgradSmem = kWarps * kSlots * (kDRow + kXRow) > 4 * kAcc * 32 * 4 + kWarps * 32 * 4
+                               ? kWarps * kSlots * (kDRow + kXRow)
+                               : 4 * kAcc * 32 * 4 + kWarps * 32 * 4;
 
 struct WgradArgs {
     const bf16 *x;
     const bf16 *dy;
-    float *dw;
-    int ldx, lddy, B, H, W, Cin, Cout, ntiles;
+    float *dw, *db;
+    int ldx, lddy, B, H, W, Cin, pieces;
 };
 
-__global__ void __launch_bounds__(288) wgrad_kernel(const WgradArgs a) {
-    __shared__ __align__(128) bf16 dyt[2][kTH * kTW * kWCo];   // [pixel][32 co], 64-byte rows
-    __shared__ __align__(128) bf16 xt[2][kPH * kPW * kWCi];    // [halo pixel][16 ci], 32-byte rows
+__global__ void __launch_bounds__(32 * kWarps, 1) wgrad_kernel(const WgradArgs a) {
+    static_assert(kItems % kSlots == 0, "static slots");
+    extern __shared__ __align__(128) unsigned char wsm[];
     const int co0 = blockIdx.x * kWCo, ci0 = blockIdx.y * kWCi;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = a.W / kTW, tiles_y = a.H / kTH;
-    const int ky = warp / 3, kx = warp % 3;  // this warp's tap
+    unsigned char *ring = wsm + warp * kSlots * (kDRow + kXRow);
+    auto dslot = [&](int s) { return reinterpret_cast<bf16 *>(ring + s * (kDRow + kXRow)); };
+    auto xslot = [&](int s) { return reinterpret_cast<bf16 *>(ring + s * (kDRow + kXRow) + kDRow); };
 
-    auto stage_in = [&](int s, int tile) {
-        const int b = tile / (tiles_x * tiles_y), r = tile % (tiles_x * tiles_y);
-        const int ty0 = (r / tiles_x) * kTH, tx0 = (r % tiles_x) * kTW;
-        for (int i = tid; i < kTH * kTW * 4; i += 288) {
-            const int pix = i >> 2, ch = i & 3;
-            const int gy = ty0 + pix / kTW, gx = tx0 + pix % kTW;
-            cp_async16(&dyt[s][sw64(pix, ch)], a.dy + ((long long)(b * a.H + gy) * a.W + gx) * a.lddy + co0 + ch * 8,
-                       16);
-        }
-        for (int i = tid; i < kPH * kPW * 2; i += 288) {
-            const int pix = i >> 1, half = i & 1;
-            const int gy = ty0 + pix / kPW - 1, gx = tx0 + pix % kPW - 1;
-            const bool in = gy >= 0 && gy < a.H && gx >= 0 && gx < a.W;
-            const bf16 *src = in ? a.x + ((long long)(b * a.H + gy) * a.W + gx) * a.ldx + ci0 + half * 8 : a.x;
-            cp_async16(&xt[s][sw32(pix, half)], src, in ? 16 : 0);
-        }
-        cp_async_commit();
+    // Piece -> image, first row, first column; pieces of one column follow one another.
+    const int rows8 = a.H / kTH, strips = a.W / kTW, stride = gridDim.z * kWarps;
+    struct Piece {
+        const bf16 *x, *dy;  // pixel (y0, x0), this block's first channel
+        int y0, x0;
     };
-
-    float acc[2][2][4];
+    auto piece_at = [&](int p) {
+        Piece r;
+        const int col = p / rows8;
+        r.y0 = (p - col * rows8) * kTH;
+        const int b = col / strips;
+        r.x0 = (col - b * strips) * kTW;
+        const long long pix = ((long long)b * a.H + r.y0) * a.W + r.x0;
+        r.x = a.x + pix * a.ldx + ci0;
+        r.dy = a.dy + pix * a.lddy + co0;
+        return r;
+    };
+    // Item i of a piece: input row y0 + i - 1 (18 pixels from x0 - 1, zeros
+    // outside the image) and, up to i = 7, output-gradient row y0 + i.
+    auto issue = [&](const Piece &r, int i) {
+        const int y = r.y0 + i - 1;
+        const bool row = y >= 0 && y < a.H;
+        bf16 *xs = xslot(i % kSlots);
 #pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 2; j++)
-#pragma unroll
-            for (int k = 0; k < 4; k++) acc[i][j][k] = 0.0f;
-
-    const int mi = lane >> 3, lr = lane & 7;
-    int s = 0;
-    int tile = blockIdx.z;
-    if (tile < a.ntiles) stage_in(0, tile);
-    for (; tile < a.ntiles; tile += gridDim.z) {
-        const int next = tile + gridDim.z;
-        if (next < a.ntiles) {
-            stage_in(s ^ 1, next);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const bf16 *D = dyt[s];
-        const bf16 *X = xt[s];
-#pragma unroll 2
-        for (int orow = 0; orow < kTH; orow++) {
-            // A (co x pixel) from the [pixel][co] tile, transposed on load:
-            // (px 0..7, co +0..7), (px 0..7, co +8..15), (px 8..15, co +0..7), (px 8..15, co +8..15)
-            uint32_t afr[2][4];
-#pragma unroll
-            for (int mt = 0; mt < 2; mt++) {
-                const int pix = orow * kTW + (mi >> 1) * 8 + lr;
-                ldsm_x4_t(afr[mt][0], afr[mt][1], afr[mt][2], afr[mt][3], &D[sw64(pix, mt * 2 + (mi & 1))]);
+        for (int h = 0; h < 2; h++) {
+            const int c = lane + 32 * h;
+            if (c < 2 * (kTW + 2)) {
+                const int px = c >> 1, half = c & 1, gx = r.x0 + px - 1;
+                const bool in = row && gx >= 0 && gx < a.W;
+                const bf16 *src = in ? r.x + ((long long)(i - 1) * a.W + px - 1) * a.ldx + half * 8 : a.x;
+                cp_async16(xs + sw32(px, half), src, in ? 16 : 0);
             }
-            // B (pixel x ci) from the halo tile at this warp's tap, transposed:
-            // (px 0..7, ci 0..7), (px 8..15, ci 0..7), (px 0..7, ci 8..15), (px 8..15, ci 8..15)
-            uint32_t bfr[2][2];
-            const int pix = (orow + ky) * kPW + (mi & 1) * 8 + lr + kx;
-            ldsm_x4_t(bfr[0][0], bfr[0][1], bfr[1][0], bfr[1][1], &X[sw32(pix, mi >> 1)]);
-#pragma unroll
-            for (int mt = 0; mt < 2; mt++)
-#pragma unroll
-                for (int nt = 0; nt < 2; nt++) mma16816(acc[mt][nt], afr[mt], bfr[nt]);
         }
-        __syncthreads();
-        s ^= 1;
-    }
-    const int g = lane >> 2, t = lane & 3;
-    const int tap = warp;
-#pragma unroll
-    for (int mt = 0; mt < 2; mt++)
-#pragma unroll
-        for (int nt = 0; nt < 2; nt++)
+        if (i < kTH) {
+            bf16 *ds = dslot(i % kSlots);
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                const int co = co0 + mt * 16 + g + h * 8, ci = ci0 + nt * 8 + 2 * t;
-                float *dst = a.dw + ((long long)co * 9 + tap) * a.Cin + ci;
-                atomicAdd(dst, acc[mt][nt][2 * h]);
-                atomicAdd(dst + 1, acc[mt][nt][2 * h + 1]);
+                const int c = lane + 32 * h, px = c >> 2, ch = c & 3;
+                cp_async16(ds + sw64(px, ch), r.dy + ((long long)i * a.W + px) * a.lddy + ch * 8, 16);
             }
-}
+        }
+    };
 
-// Bias gradient: db[co] += sum over pixels of dy[., co].
-__global__ void bias_grad_kernel(const bf16 *dy, int lddy, long long P, int C, float *db) {
-    const long long per = (P + gridDim.x - 1) / gridDim.x;
-    const long long p0 = blockIdx.x * per, p1 = p0 + per < P ? p0 + per : P;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float s = 0.0f;
-        for (long long p = p0; p < p1; p++) s += __bfloat162float(dy[p * lddy + c]);
-        atomicAdd(db + c, s);
+    float acc[9][2][2][4];
+    float bsum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int t = 0; t < 9; t++)
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+#pragma unroll
+            for (int j = 0; j < 2; j++)
+#pragma unroll
+                for (int k = 0; k < 4; k++) acc[t][i][j][k] = 0.0f;
+
+    const int mi = lane >> 3, lr = lane & 7;
+    int p = blockIdx.z * kWarps + warp;
+    Piece cur = piece_at(p < a.pieces ? p : 0), nxt = cur;
+#pragma unroll
+    for (int i = 0; i < kSlots - 1; i++) {
+        if (p < a.pieces) issue(cur, i);
+        cp_async_commit();
+    }
+    uint32_t afr[3][2][4];  // output-gradient fragments of the last three rows
+    for (; p < a.pieces; p += stride) {
+        const bool more = p + stride < a.pieces;
+        if (more) nxt = piece_at(p + stride);
+        const bool bias = a.db && p % (int)gridDim.y == (int)blockIdx.y;
+#pragma unroll
+        for (int i = 0; i < kItems; i++) {
+            cp_async_wait<kSlots - 2>();  // item i has landed
+            __syncwarp();
+            if (i < kTH) {
+                // A (co x pixel), transposed on load: (px 0..7, co +0..7),
+                // (px 0..7, co +8..15), (px 8..15, co +0..7), (px 8..15, co +8..15)
+                const bf16 *D = dslot(i % kSlots);
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++) {
+                    uint32_t *f = afr[i % 3][mt];
+                    ldsm_x4_t(f[0], f[1], f[2], f[3], D + sw64((mi >> 1) * 8 + lr, mt * 2 + (mi & 1)));
+                }
+            }
+            // B (pixel x ci) at the three horizontal shifts, transposed on load:
+            // (px 0..7, ci 0..7), (px 8..15, ci 0..7), (px 0..7, ci 8..15), (px 8..15, ci 8..15)
+            const bf16 *X = xslot(i % kSlots);
+            uint32_t bfr[3][4];
+#pragma unroll
+            for (int kx = 0; kx < 3; kx++)
+                ldsm_x4_t(bfr[kx][0], bfr[kx][1], bfr[kx][2], bfr[kx][3], X + sw32((mi & 1) * 8 + lr + kx, mi >> 1));
+            // the slot read one item ago takes the item four ahead
+            const int ahead = i + kSlots - 1;
+            if (ahead < kItems) issue(cur, ahead);
+            else if (more) issue(nxt, ahead - kItems);
+            cp_async_commit();
+            if (i < kTH && bias) {
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const uint32_t q = afr[i % 3][mt][h], r = afr[i % 3][mt][h + 2];
+                        bsum[2 * mt + h] += (__uint_as_float(q << 16) + __uint_as_float(q & 0xffff0000u)) +
+                                            (__uint_as_float(r << 16) + __uint_as_float(r & 0xffff0000u));
+                    }
+            }
+            // input row y0 + i - 1 meets output rows y0 + i - ky at tap row ky
+#pragma unroll
+            for (int ky = 0; ky < 3; ky++)
+                if (i - ky >= 0 && i - ky < kTH) {
+#pragma unroll
+                    for (int kx = 0; kx < 3; kx++)
+#pragma unroll
+                        for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+                            for (int nt = 0; nt < 2; nt++)
+                                mma16816(acc[3 * ky + kx][mt][nt], afr[(i - ky + 3) % 3][mt], bfr[kx] + 2 * nt);
+                }
+        }
+        cur = nxt;
+    }
+    // Fold the eight warps' sums: the upper four into the lower four, then four
+    // areas element by element; one atomic per weight and block.
+    cp_async_wait<0>();
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(wsm);
+    float *bred = red + 4 * kAcc * 32;
+    auto each = [&](auto f) {
+#pragma unroll
+        for (int t = 0; t < 9; t++)
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int j = 0; j < 2; j++)
+#pragma unroll
+                    for (int k = 0; k < 4; k++) f(((t * 2 + i) * 2 + j) * 4 + k, acc[t][i][j][k]);
+    };
+    float *mine = red + (warp & 3) * kAcc * 32 + lane;
+    if (warp >= 4) each([&](int e, float &v) { mine[e * 32] = v; });
+    // co = 16 mt + 8 h + lane / 4; the four lanes of a co hold different pixels
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        bsum[k] += __shfl_xor_sync(0xffffffffu, bsum[k], 1);
+        bsum[k] += __shfl_xor_sync(0xffffffffu, bsum[k], 2);
+        if ((lane & 3) == 0) bred[warp * 32 + (k >> 1) * 16 + (k & 1) * 8 + (lane >> 2)] = bsum[k];
+    }
+    __syncthreads();
+    if (warp < 4) each([&](int e, float &v) { mine[e * 32] += v; });
+    __syncthreads();
+    for (int e = tid; e < kAcc * 32; e += 32 * kWarps) {
+        const float v = (red[e] + red[e + kAcc * 32]) + (red[e + 2 * kAcc * 32] + red[e + 3 * kAcc * 32]);
+        const int l = e & 31, q = e >> 5, k = q & 3, j = (q >> 2) & 1, i = (q >> 3) & 1, t = q >> 4;
+        const int co = co0 + i * 16 + (l >> 2) + (k >> 1) * 8, ci = ci0 + j * 8 + 2 * (l & 3) + (k & 1);
+        atomicAdd(a.dw + ((long long)co * 9 + t) * a.Cin + ci, v);
+    }
+    if (a.db && tid < kWCo) {
+        float v = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kWarps; w++) v += bred[w * 32 + tid];
+        atomicAdd(a.db + co0 + tid, v);
     }
 }
 
@@ -689,21 +782,19 @@ int lbmfvm_sg_conv3x3_wgrad(const uint16_t *x, int32_t ldx, const uint16_t *dy, 
         return sg_fail(kErrArg, "wgrad: shape B=%d H=%d W=%d Cin=%d Cout=%d breaks the tile rules", B, H, W, Cin, Cout);
     if (ldx < Cin || lddy < Cout || ldx % 8 || lddy % 8 || !aligned16(x) || !aligned16(dy))
         return sg_fail(kErrArg, "wgrad: strides or alignment");
-    const int ntiles = B * (H / kTH) * (W / kTW);
+    const int pieces = B * (H / kTH) * (W / kTW);
     const int gx = Cout / kWCo, gy = Cin / kWCi;
-    int split = (4 * 152 + gx * gy - 1) / (gx * gy);
-    split = split < ntiles ? split : ntiles;
-    WgradArgs a{reinterpret_cast<const bf16 *>(x), reinterpret_cast<const bf16 *>(dy), dw, ldx, lddy, B, H, W, Cin,
-                Cout, ntiles};
-    wgrad_kernel<<<dim3(gx, gy, split), 288, 0, (cudaStream_t)stream>>>(a);
-    if (int r = launched("wgrad")) return r;
-    if (db) {
-        const long long P = (long long)B * H * W;
-        bias_grad_kernel<<<grid_for(P, 1024) < 512 ? grid_for(P, 1024) : 512, 128, 0, (cudaStream_t)stream>>>(
-            reinterpret_cast<const bf16 *>(dy), lddy, P, Cout, db);
-        return launched("bias gradient");
-    }
-    return kOk;
+    // one block per SM (the accumulators fill its registers), fewer where the
+    // pieces would not give every warp one
+    int split = 152 / (gx * gy);
+    if (split < 1) split = 1;
+    if (split > (pieces + kWarps - 1) / kWarps) split = (pieces + kWarps - 1) / kWarps;
+    WgradArgs a{reinterpret_cast<const bf16 *>(x), reinterpret_cast<const bf16 *>(dy), dw, db, ldx, lddy, B, H, W, Cin,
+                pieces};
+    const cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgradSmem);
+    if (e != cudaSuccess) return sg_fail(kErrCuda, "wgrad: %s", cudaGetErrorString(e));
+    wgrad_kernel<<<dim3(gx, gy, split), 32 * kWarps, kWgradSmem, (cudaStream_t)stream>>>(a);
+    return launched("wgrad");
 }
 
 int lbmfvm_sg_pool2(const uint16_t *x, int32_t ldx, uint16_t *y, int32_t ldy, int32_t B, int32_t H, int32_t W,

@@ -91,3 +91,32 @@ def test_output_layer_over_its_forms(P, C, CO, pad):
     assert np.abs(h(dxv).reshape(P, C) - ref).max() <= 2.0 ** -8 * np.abs(ref).max()
     if pad:
         assert not dxt[..., :pad].any() and not dxt[..., pad + C:].any()
+
+
+# one piece of 8 x 16 pixels; fewer pieces than a block has warps; pieces that do not fill the last round; sliced
+# channels; the widest layer's 160 x 160; with and without the bias gradient
+@pytest.mark.parametrize("B,H,W,cin,cout,pad,bias", [(1, 8, 16, 16, 32, 0, True), (1, 24, 16, 48, 64, 8, True),
+                                                     (3, 16, 48, 32, 32, 8, False), (5, 16, 16, 160, 160, 0, True),
+                                                     (2, 128, 128, 96, 32, 0, True), (1, 64, 240, 16, 96, 16, True)])
+def test_weight_and_bias_gradient_over_their_shapes(B, H, W, cin, cout, pad, bias):
+    rng = np.random.default_rng(B + H + W + cin + cout)
+    xt, xv, xp, ldx = slice_of(rand(rng, B, H, W, cin), pad)
+    dt, dv, dp, ldd = slice_of(rand(rng, B, H, W, cout), pad)
+    if pad:  # what lies beside the slices is not read
+        for t, c in ((xt, cin), (dt, cout)):
+            t[..., :pad] = t[..., pad + c:] = float("nan")
+    dw, db = torch.ones(cout, 9, cin, device="cuda"), torch.ones(cout, device="cuda")
+    S.call("lbmfvm_sg_conv3x3_wgrad", xp, ldx, dp, ldd, dw.data_ptr(), db.data_ptr() if bias else None, B, H, W, cin,
+           cout, S._stream())
+    torch.cuda.synchronize()
+    x, dy = xv.double(), dv.double().reshape(-1, cout)
+    xpad = torch.nn.functional.pad(x, (0, 0, 1, 1, 1, 1))
+    taps = [xpad[:, k // 3:k // 3 + H, k % 3:k % 3 + W].reshape(-1, cin) for k in range(9)]
+    want = torch.stack([dy.t() @ t for t in taps], 1)
+    size = torch.stack([dy.abs().t() @ t.abs() for t in taps], 1)
+    # FP32 sums of exact BF16 products: a warp's chain is some hundred terms, so 64 ulp of the sum of sizes is ample
+    assert bool(((dw.double() - 1 - want).abs() <= 64 * 2.0 ** -23 * (size + 1)).all())
+    if bias:
+        assert bool(((db.double() - 1 - dy.sum(0)).abs() <= 64 * 2.0 ** -23 * (dy.abs().sum(0) + 1)).all())
+    else:
+        assert bool((db == 1).all())
