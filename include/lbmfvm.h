@@ -3,8 +3,8 @@
  * for natural convection: the hybrid LBM(velocity) + FVM(temperature) method
  * of Li, Yang & Zhang, arXiv 1908.08386, Section 5.
  *
- * One time step of a handle is one launch of a fused CUDA kernel that, per
- * node,
+ * One time step of a handle is one launch of a fused CUDA kernel (or a pass of a
+ * launch that takes many steps, see LBMFVM_KERNEL_AUTO) that, per node,
  *   - pulls the post-collision D2Q9 populations of the previous step from the
  *     neighbours (Eq. 5, velocity set of Eq. 4, weights of Eq. 9);
  *   - rebuilds wall nodes by non-equilibrium extrapolation from their inner
@@ -79,7 +79,13 @@ extern "C" {
  *            storage type);
  *   GENERIC  one block per tile, gathers straight from global memory (any
  *            boundary, every storage type).
- * AUTO takes TMA where it applies and GENERIC otherwise. */
+ * AUTO takes TMA where it applies and GENERIC otherwise; with a tile shape left
+ * to the library too (tma_config TMA_DEFAULT or TMA_AUTOTUNE), grids and batches
+ * whose tiles fit the SMs one per block (up to about 300,000 nodes in FP32, 75,000
+ * in 64-bit types) run all but the last of eight or more steps of a call in one
+ * launch that keeps the state on the chip, with the same results.  Such launches
+ * of one process go one after another on a device, and are not taken while the
+ * stream is being captured. */
 #define LBMFVM_KERNEL_AUTO 0
 #define LBMFVM_KERNEL_GENERIC 1
 #define LBMFVM_KERNEL_TMA 2
@@ -323,8 +329,10 @@ int lbmfvm_run_to_steady(lbmfvm_t *h, double tol, int64_t check_every, int64_t m
  * after src's queued work. */
 int lbmfvm_copy_state(lbmfvm_t *dst, lbmfvm_t *src);
 
-/* Number of step-kernel launches lbmfvm_step has issued on this handle (one
- * per coupled step; a CUDA-graph replay counts the launches it holds). */
+/* Number of coupled steps lbmfvm_step has issued to step kernels on this handle
+ * (one launch per step; a CUDA-graph replay counts the launches it holds, and a
+ * resident launch, which keeps a small grid on the chip over many steps, counts
+ * the steps it takes). */
 int lbmfvm_launch_count(const lbmfvm_t *h, int64_t *launches);
 
 /* Step kernel in use (LBMFVM_KERNEL_TMA or LBMFVM_KERNEL_GENERIC) and the TMA

@@ -306,11 +306,13 @@ __device__ __forceinline__ void collide(const C g[9], C drho, C ux, C uy, C omeg
 template <class C>
 __device__ __forceinline__ C fv_update(C TP, C uP, C vP, C ex, C ey, C alpha, bool oE, C TE, C uE, bool oN, C TN,
                                        C vN, bool oW, C TW, C uW, bool oS, C TS, C vS) {
+    // the diffusive product joins the rounded advective one in one fused
+    // multiply-add, whichever kernel this is compiled into
     const C q = C(0.25);
-    const C fe = oE ? alpha * (TE - TP) - q * (uP + uE) * (TP + TE) : C(0);
-    const C fw = oW ? alpha * (TW - TP) + q * (uP + uW) * (TP + TW) : C(0);
-    const C fn = oN ? alpha * (TN - TP) - q * (vP + vN) * (TP + TN) : C(0);
-    const C fs = oS ? alpha * (TS - TP) + q * (vP + vS) * (TP + TS) : C(0);
+    const C fe = oE ? fma_c(alpha, TE - TP, -mul_r(q * (uP + uE), TP + TE)) : C(0);
+    const C fw = oW ? fma_c(alpha, TW - TP, mul_r(q * (uP + uW), TP + TW)) : C(0);
+    const C fn = oN ? fma_c(alpha, TN - TP, -mul_r(q * (vP + vN), TP + TN)) : C(0);
+    const C fs = oS ? fma_c(alpha, TS - TP, mul_r(q * (vP + vS), TP + TS)) : C(0);
     // 1/(ex ey) is a power of two (ex, ey in {1/2, 1}): the product is exact.
     const C inv_v = (ex < C(1) ? C(2) : C(1)) * (ey < C(1) ? C(2) : C(1));
     return TP + (ey * (fe + fw) + ex * (fn + fs)) * inv_v;
@@ -326,9 +328,9 @@ __device__ __forceinline__ C fv_update(C TP, C uP, C vP, C ex, C ey, C alpha, bo
 template <class C>
 __device__ __forceinline__ C quick_face(C un, C TP, C Tn, bool farP, C TfarP, bool farN, C TfarN) {
     if (!(un < C(0))) {
-        if (farP) return C(0.75) * TP + C(0.375) * Tn - C(0.125) * TfarP;
+        if (farP) return fma_c(C(0.75), TP, mul_r(C(0.375), Tn)) - C(0.125) * TfarP;
     } else if (farN) {
-        return C(0.75) * Tn + C(0.375) * TP - C(0.125) * TfarN;
+        return fma_c(C(0.375), TP, mul_r(C(0.75), Tn)) - C(0.125) * TfarN;
     }
     return C(0.5) * (TP + Tn);
 }
@@ -342,12 +344,12 @@ __device__ __forceinline__ C fv_update_faces(C TP, C uP, C vP, C ex, C ey, C alp
                                              bool oN, C TN, C vN, C TfN, bool oW, C TW, C uW, C TfW, bool oS, C TS,
                                              C vS, C TfS) {
     const C h = C(0.5);
-    const C fe = oE ? alpha * (TE - TP) - h * (uP + uE) * TfE : C(0);
-    const C fw = oW ? alpha * (TW - TP) + h * (uP + uW) * TfW : C(0);
-    const C fn = oN ? alpha * (TN - TP) - h * (vP + vN) * TfN : C(0);
-    const C fs = oS ? alpha * (TS - TP) + h * (vP + vS) * TfS : C(0);
+    const C fe = oE ? fma_c(alpha, TE - TP, -mul_r(h * (uP + uE), TfE)) : C(0);
+    const C fw = oW ? fma_c(alpha, TW - TP, mul_r(h * (uP + uW), TfW)) : C(0);
+    const C fn = oN ? fma_c(alpha, TN - TP, -mul_r(h * (vP + vN), TfN)) : C(0);
+    const C fs = oS ? fma_c(alpha, TS - TP, mul_r(h * (vP + vS), TfS)) : C(0);
     const C inv_v = (ex < C(1) ? C(2) : C(1)) * (ey < C(1) ? C(2) : C(1));
-    return TP + dt * ((ey * (fe + fw) + ex * (fn + fs)) * inv_v);
+    return fma_c(dt, (ey * (fe + fw) + ex * (fn + fs)) * inv_v, TP);
 }
 
 __host__ __device__ __forceinline__ bool fv_open(uint8_t code) { return (code >> 6) <= TH_DIRICHLET; }
@@ -1113,7 +1115,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                 Tn = TT[tidx(lx + cx_rt(d), ly + cy_rt(d))];
             }
             OT[ly * TW + lx] = Tn;
-            const C Gy = fy + gbeta * (Tn - t_ref);
+            const C Gy = fma_c(gbeta, Tn - t_ref, fy);
             collide<C>(g[j], dr[j], uu[j], vv[j], omega, fx, Gy, [&](int q, C v) { st(of + q * OPLANE, v); });
         }
         if (tid == PROD && k > 0 && pre_t >= 0) {

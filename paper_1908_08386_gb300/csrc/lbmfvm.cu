@@ -24,12 +24,18 @@
 
 #include "kernels.cuh"
 #include "lbmfvm.h"
+#include "resident.cuh"
 
 using namespace lbmfvm_dev;
 
 namespace {
 
 constexpr int kGraphSteps = 64;      // launches per captured graph (even)
+// Steps from which a resident launch is worth it: it loads and stores the
+// state once (about 8 us with the launch) and saves 1.4 us or more a step
+// (9 steps of 64^2 FP32: 22.7 us against 39.4; of 512^2: 68.6 against 74.7).
+constexpr int kResidentMin = 8;
+constexpr int kResidentSteps = 1 << 16;  // steps of one resident launch at most
 constexpr int kResidualBlocks = 608; // 4 x 152 SMs
 // Reduction scratch (doubles): kResidualSums partials per residual block,
 // then the totals, the wall temperatures of the initial state, the two mean
@@ -79,9 +85,31 @@ struct Layout {
     size_t uv[2], tx[2];
     bool split;
     size_t g[2];  // D2Q5 energy populations [5][ny][pitch] (0 for the FV energy update)
+    // resident launches: tile headers and mailboxes (mail_bytes 0: none fit)
+    size_t rtiles, mail, mail_bytes;
 };
 
-Layout make_layout(const lbmfvm_grid_t &g, int prec, int ncav = 1, bool split = false, bool lbm5 = false) {
+// Resident launches (resident.cuh) hold one tile per SM.
+constexpr int kResidentSlots = 152;
+
+lbmfvm_fv::ResShape res_shape(int prec, int i) {
+    switch (prec) {
+        case LBMFVM_F64: return lbmfvm_fv::resident_shape<double>(i);
+        case LBMFVM_F16: return lbmfvm_fv::resident_shape<__half>(i);
+        case LBMFVM_BF16: return lbmfvm_fv::resident_shape<__nv_bfloat16>(i);
+        case LBMFVM_F32X2: return lbmfvm_fv::resident_shape<dsf>(i);
+        default: return lbmfvm_fv::resident_shape<float>(i);
+    }
+}
+
+long long res_tiles_of(const lbmfvm_fv::ResShape &s, int nx, int ny) {
+    return (long long)((nx + s.TW - 1) / s.TW) * ((ny + s.TH - 1) / s.TH);
+}
+
+// ncav: cavities of a batch's packed grid (0: a single cavity).
+Layout make_layout(const lbmfvm_grid_t &g, int prec, int ncav, bool split, bool lbm5) {
+    const bool batch = ncav > 0;
+    ncav = batch ? ncav : 1;
     Layout L{};
     L.pitch = (int)align_up((size_t)g.nx, 64);
     L.plane = (long long)g.ny * L.pitch;
@@ -120,6 +148,19 @@ Layout make_layout(const lbmfvm_grid_t &g, int prec, int ncav = 1, bool split = 
     L.tile_cap = max_tiles;
     // two lists (fused step; sub-step path), each a count slot and its headers
     L.tiles = take((max_tiles + 2) * sizeof(TileHeader));
+    // resident launches: what the largest need of any shape that fits is (a
+    // batch may shrink to any of them as its cavities converge)
+    const bool periodic = g.bc[LBMFVM_SIDE_W] == LBMFVM_BC_PERIODIC || g.bc[LBMFVM_SIDE_S] == LBMFVM_BC_PERIODIC;
+    for (int i = 0; i < kResShapes && !periodic; i++) {
+        const lbmfvm_fv::ResShape s = res_shape(prec, i);
+        if (!s.TW) continue;
+        const long long tiles = batch ? kResidentSlots : res_tiles_of(s, g.nx, g.ny);
+        if (tiles <= kResidentSlots) L.mail_bytes = std::max(L.mail_bytes, (size_t)tiles * s.mail_bytes);
+    }
+    if (L.mail_bytes) {
+        L.rtiles = take(kResidentSlots * sizeof(TileHeader));
+        L.mail = take(L.mail_bytes);
+    }
     L.total = off;
     return L;
 }
@@ -293,6 +334,10 @@ struct lbmfvm {
     int fv_every;                    // lattice steps per coarse energy step
     int ncx, ncy;                    // coarse volumes
     uint64_t tiles_gen, graph_gen;   // tile-list generation, and the one the graph was captured with
+    bool res_allowed;                // kernel and tile shape are the library's choice
+    int res_shape, res_tiles;        // shape of resident launches (-1: none fits the active tiles) and its tiles
+    bool res_general;                // they take the general energy update (QUICK or sub-steps)
+    uint32_t res_seq;                // exchanges made since the resident tile list was built
     uint32_t code_crc; // CRC-32 of the node codes, identifies the geometry in checkpoints
     int tile_w, tile_h;
     // Several cavities packed in one grid (batch handles); empty for one cavity.
@@ -803,6 +848,96 @@ int setup_tma(lbmfvm_t *h) {
     return upload_tiles(h, g.TW, g.TH);
 }
 
+// Header of the tile of cavity c (descriptor cd) at (x0, y0).
+TileHeader tile_header(const CavityDesc &cd, int c, int x0, int y0) {
+    const int m = cd.substeps < 1 ? 1 : cd.substeps;
+    TileHeader t{};
+    t.x0 = x0;
+    t.y0 = y0;
+    t.ox = x0 - cd.x0;
+    t.oy = y0 - cd.y0;
+    t.nx = cd.nx;
+    t.ny = cd.ny;
+    t.cav = c;
+    t.substeps = m;
+    t.omega = cd.omega;
+    t.alpha = cd.alpha;
+    t.gbeta = cd.gbeta;
+    t.t_ref = cd.t_ref;
+    t.fx = cd.fx;
+    t.fy = cd.fy;
+    t.omega_f = (float)cd.omega;
+    t.alpha_f = (float)cd.alpha;
+    t.gbeta_f = (float)cd.gbeta;
+    t.t_ref_f = (float)cd.t_ref;
+    t.fx_f = (float)cd.fx;
+    t.fy_f = (float)cd.fy;
+    const double dt = 1.0 / m;
+    t.dt_f = (float)dt;
+    auto lo = [](double d) { return (float)(d - (double)(float)d); };
+    t.omega_lo = lo(cd.omega);
+    t.alpha_lo = lo(cd.alpha);
+    t.gbeta_lo = lo(cd.gbeta);
+    t.t_ref_lo = lo(cd.t_ref);
+    t.fx_lo = lo(cd.fx);
+    t.fy_lo = lo(cd.fy);
+    t.dt_lo = lo(dt);
+    return t;
+}
+
+// Blocks per SM of resident shape i for the handle's storage.
+cudaError_t res_prepare(const lbmfvm_t *h, int i, bool general, int *blocks) {
+    switch (h->prec) {
+        case LBMFVM_F64: return lbmfvm_fv::resident_prepare<double>(i, general, blocks);
+        case LBMFVM_F16: return lbmfvm_fv::resident_prepare<__half>(i, general, blocks);
+        case LBMFVM_BF16: return lbmfvm_fv::resident_prepare<__nv_bfloat16>(i, general, blocks);
+        case LBMFVM_F32X2: return lbmfvm_fv::resident_prepare<dsf>(i, general, blocks);
+        default: return lbmfvm_fv::resident_prepare<float>(i, general, blocks);
+    }
+}
+
+// The resident launches' tile list: the smallest shape whose tiles over the
+// active cavities fit one per SM, if any.  A new list starts with cleared
+// mailboxes, so that no tag of an earlier list can be taken for one of its own.
+int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
+    h->res_shape = -1;
+    h->res_tiles = 0;
+    if (!h->res_allowed || !h->L.mail_bytes || h->grid2) return LBMFVM_OK;
+    const int slots = std::min(kResidentSlots, h->num_sms);
+    auto active = [&](size_t c) { return h->atlas_cavs.empty() || h->atlas_active[c]; };
+    h->res_general = h->fv_quick;
+    for (size_t c = 0; c < table.size(); c++)
+        if (active(c) && table[c].substeps > 1) h->res_general = true;
+    std::vector<TileHeader> list;
+    for (int i = 0; i < kResShapes; i++) {
+        const lbmfvm_fv::ResShape sh = res_shape(h->prec, i);
+        if (!sh.TW) continue;
+        long long tiles = 0;
+        for (size_t c = 0; c < table.size(); c++)
+            if (active(c)) tiles += res_tiles_of(sh, table[c].nx, table[c].ny);
+        if (tiles < 1 || tiles > slots || (size_t)tiles * sh.mail_bytes > h->L.mail_bytes) continue;
+        int blocks = 0;
+        CU(h, res_prepare(h, i, h->res_general, &blocks));
+        if (blocks < 1) continue;
+        for (size_t c = 0; c < table.size(); c++) {
+            if (!active(c)) continue;
+            const CavityDesc &cd = table[c];
+            for (int y0 = cd.y0; y0 < cd.y0 + cd.ny; y0 += sh.TH)
+                for (int x0 = cd.x0; x0 < cd.x0 + cd.nx; x0 += sh.TW)
+                    list.push_back(tile_header(cd, (int)c, x0, y0));
+        }
+        h->res_shape = i;
+        h->res_tiles = (int)tiles;
+        h->res_seq = 0;
+        CU(h, cudaMemsetAsync(h->base + h->L.mail, 0, (size_t)tiles * sh.mail_bytes, h->s));
+        CU(h, cudaMemcpyAsync(h->base + h->L.rtiles, list.data(), list.size() * sizeof(TileHeader),
+                              cudaMemcpyHostToDevice, h->s));
+        break;
+    }
+    CU(h, cudaStreamSynchronize(h->s));  // the list is the host's
+    return LBMFVM_OK;
+}
+
 // Tile lists of the TMA kernel (row by row over every active cavity) and the
 // cavity table, uploaded on the handle's stream: cavities with one energy
 // update per step in the fused list, those with sub-steps in the second list,
@@ -825,38 +960,7 @@ int upload_tiles(lbmfvm_t *h, int tw, int th) {
         std::vector<TileHeader> &tl = m > 1 || h->grid2 ? split : fused;
         for (int y0 = cd.y0; y0 < cd.y0 + cd.ny; y0 += th)
             for (int x0 = cd.x0; x0 < cd.x0 + cd.nx; x0 += tw) {
-                TileHeader t{};
-                t.x0 = x0;
-                t.y0 = y0;
-                t.ox = x0 - cd.x0;
-                t.oy = y0 - cd.y0;
-                t.nx = cd.nx;
-                t.ny = cd.ny;
-                t.cav = (int)c;
-                t.substeps = m;
-                t.omega = cd.omega;
-                t.alpha = cd.alpha;
-                t.gbeta = cd.gbeta;
-                t.t_ref = cd.t_ref;
-                t.fx = cd.fx;
-                t.fy = cd.fy;
-                t.omega_f = (float)cd.omega;
-                t.alpha_f = (float)cd.alpha;
-                t.gbeta_f = (float)cd.gbeta;
-                t.t_ref_f = (float)cd.t_ref;
-                t.fx_f = (float)cd.fx;
-                t.fy_f = (float)cd.fy;
-                const double dt = 1.0 / m;
-                t.dt_f = (float)dt;
-                auto lo = [](double d) { return (float)(d - (double)(float)d); };
-                t.omega_lo = lo(cd.omega);
-                t.alpha_lo = lo(cd.alpha);
-                t.gbeta_lo = lo(cd.gbeta);
-                t.t_ref_lo = lo(cd.t_ref);
-                t.fx_lo = lo(cd.fx);
-                t.fy_lo = lo(cd.fy);
-                t.dt_lo = lo(dt);
-                tl.push_back(t);
+                tl.push_back(tile_header(cd, (int)c, x0, y0));
             }
     }
     if (!split.empty() && !h->L.split)
@@ -888,7 +992,7 @@ int upload_tiles(lbmfvm_t *h, int tw, int th) {
     CU(h, cudaMemcpyAsync(h->base + h->L.cav, table.data(), table.size() * sizeof(CavityDesc),
                           cudaMemcpyHostToDevice, h->s));
     CU(h, cudaStreamSynchronize(h->s));
-    return LBMFVM_OK;
+    return upload_resident(h, table);
 }
 
 // Clears the tile counters of both lists (a step of parity p clears the
@@ -1195,7 +1299,7 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
     if (fv_opt && (!tma_ok || opts.kernel == LBMFVM_KERNEL_GENERIC))
         return fail_thread(LBMFVM_ERR_ARG, "QUICK face values and energy sub-steps need the TMA kernel (walls on every side)");
     if (atlas && !tma_ok) return fail_thread(LBMFVM_ERR_ARG, "a batch needs walls on every side");
-    const Layout L = make_layout(*grid, opts.store, atlas ? (int)atlas->cavs.size() : 1, split, lbm5);
+    const Layout L = make_layout(*grid, opts.store, atlas ? (int)atlas->cavs.size() : 0, split, lbm5);
     if (opts.workspace && opts.workspace_bytes < L.total)
         return fail_thread(LBMFVM_ERR_NOMEM, "workspace of %zu bytes is smaller than the %zu needed",
                            opts.workspace_bytes, L.total);
@@ -1233,8 +1337,12 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
             shape_default = small ? 2 : state <= (size_t)l2 ? 4 : 5;
         }
     }
-    h->tma_config = opts.tma_config == LBMFVM_TMA_AUTOTUNE || opts.tma_config == LBMFVM_TMA_DEFAULT ? shape_default
-                                                                                                  : opts.tma_config;
+    const bool own_shape = opts.tma_config == LBMFVM_TMA_AUTOTUNE || opts.tma_config == LBMFVM_TMA_DEFAULT;
+    h->tma_config = own_shape ? shape_default : opts.tma_config;
+    // a handle (or batch) whose kernel and tile shape are left to the library
+    // may run many steps per launch (resident.cuh)
+    h->res_allowed = own_shape && (atlas || opts.kernel == LBMFVM_KERNEL_AUTO);
+    h->res_shape = -1;
     h->fv_quick = opts.fv_scheme == LBMFVM_FV_QUICK;
     h->fv_sub = m;
     h->energy = opts.energy;
@@ -1334,9 +1442,79 @@ int fields_impl(lbmfvm_t *h, O *rho, O *u, O *v, O *T) {
 }  // namespace
 
 namespace {
+// Resident launches of one device go one after another: the blocks of two of
+// them that each got part of the SMs would wait for their missing ones.  The
+// last launch's event orders the next one, whichever handle, stream or thread
+// it comes from.
+struct ResidentGate {
+    std::mutex mu;
+    cudaEvent_t last[64] = {};
+};
+ResidentGate g_resident;
+
+// Whether n steps from now may go into resident launches: enough of them to
+// pay for the launch (loading and storing the state), nothing injected, and
+// no capture by the caller (tags count on, so a launch cannot be replayed).
+bool resident_steps(lbmfvm_t *h, int64_t n) {
+    if (h->res_shape < 0 || h->stall_next || n < kResidentMin) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(h->s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+}
+
+// n steps in one resident launch (both population buffers and temperature
+// planes hold the state's two last steps only after one more ordinary step).
+template <class S>
+int launch_resident(lbmfvm_t *h, int n) {
+    ResArgs<S> r{};
+    r.a = args_for<S>(h, h->parity);
+    r.fflags = h->base + h->L.fflags;
+    r.cavs = reinterpret_cast<const CavityDesc *>(h->base + h->L.cav);
+    r.tiles = reinterpret_cast<const TileHeader *>(h->base + h->L.rtiles);
+    r.mailbox = reinterpret_cast<uint64_t *>(h->base + h->L.mail);
+    r.seq0 = h->res_seq;
+    r.nsteps = n;
+    r.quick = h->fv_quick;
+    r.tile_w = h->tile_w;
+    r.tile_h = h->tile_h;
+    r.ctr[0] = reinterpret_cast<int *>(h->base + list_fused(h).slot) + 1;
+    r.ctr[1] = reinterpret_cast<int *>(h->base + list_split(h).slot) + 1;
+    int dev = 0;
+    CU(h, cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return fail(h, LBMFVM_ERR_CUDA, "device %d", dev);
+    std::lock_guard<std::mutex> lock(g_resident.mu);
+    cudaEvent_t &last = g_resident.last[dev];
+    if (!last) CU(h, cudaEventCreateWithFlags(&last, cudaEventDisableTiming));
+    else CU(h, cudaStreamWaitEvent(h->s, last, 0));
+    CU(h, lbmfvm_fv::resident_launch<S>(h->res_shape, h->res_general, r, h->res_tiles, h->s));
+    CU(h, cudaEventRecord(last, h->s));
+    h->res_seq += (uint32_t)n;
+    h->parity ^= 1;
+    h->steps += n;
+    h->launches += n;
+    return LBMFVM_OK;
+}
+
+int run_resident(lbmfvm_t *h, int n) {
+    switch (h->prec) {
+        case LBMFVM_F64: return launch_resident<double>(h, n);
+        case LBMFVM_F32: return launch_resident<float>(h, n);
+        case LBMFVM_F16: return launch_resident<__half>(h, n);
+        case LBMFVM_BF16: return launch_resident<__nv_bfloat16>(h, n);
+        case LBMFVM_F32X2: return launch_resident<dsf>(h, n);
+    }
+    return LBMFVM_OK;
+}
+
 // lbmfvm_step without the joins with the caller's stream: the launches of
 // n steps on the handle's own stream.
 int step_impl(lbmfvm_t *h, int64_t n) {
+    if (resident_steps(h, n)) {
+        while (n > 1) {
+            const int k = (int)std::min<int64_t>(n - 1, kResidentSteps);
+            if (int r = run_resident(h, k)) return r;
+            n -= k;
+        }
+    }
     // tile lists that changed since the capture need other grids and
     // sub-step launches
     if (h->graph && h->use_tma && h->graph_gen != h->tiles_gen) {
@@ -1391,7 +1569,7 @@ int lbmfvm_workspace_bytes(const lbmfvm_grid_t *grid, const lbmfvm_opts_t *opts,
     // sub-steps (or the automatic choice, which may take them) need the planes
     const bool split = opts && (opts->fv_substeps != 1 || opts->fv_grid == 2);
     const bool lbm5 = opts && opts->energy == LBMFVM_ENERGY_LBM_D2Q5;
-    *bytes = make_layout(*grid, prec, 1, split, lbm5).total;
+    *bytes = make_layout(*grid, prec, 0, split, lbm5).total;
     return LBMFVM_OK;
 }
 
