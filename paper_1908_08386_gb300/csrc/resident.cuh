@@ -8,8 +8,8 @@
 // drain, which bound small cavities whatever their size.  Measured (us per
 // step, one launch per step -> resident): FP32 64^2 3.68 -> 1.68, 128^2 3.98 ->
 // 1.89, 256^2 4.62 -> 2.16, 384^2 4.93 -> 3.19, 512^2 7.55 -> 5.89; FP16 256^2
-// 4.45 -> 2.28; double-single 64^2 7.05 -> 5.42, 128^2 7.15 -> 5.56, 192^2 7.95 ->
-// 5.41, 256^2 11.0 -> 9.7; FP64 64^2 21.0 -> 9.3, 128^2 21.0 -> 11.7, 192^2 21.1 ->
+// 4.45 -> 2.28; double-single 64^2 5.82 -> 3.39, 128^2 5.76 -> 3.04, 192^2 5.95 ->
+// 3.57, 256^2 8.5 -> 6.3; FP64 64^2 21.0 -> 9.3, 128^2 21.0 -> 11.7, 192^2 21.1 ->
 // 19.3; 512 x 384 with QUICK and two sub-steps (four launches) 27.2 -> 10.3.
 // What bounds it now: the exchange (about 1.1 us) and, for the 64-bit types,
 // the dependent chain of one node's operations.
@@ -456,15 +456,16 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                 const int i = tid + j * G::NT, ly = i / TW, lx = i - ly * TW;
                 const uint32_t c = info[j];
                 const int kind = c & 3;
-                if (kind == KIND_FLUID) {
-                    pull(lx, ly, g[j]);
-                    moments<C>(g[j], dr[j], uu[j], vv[j]);
-                } else if (kind == KIND_WALL) {
-                    const int d = partner_dir((uint8_t)c);
+                if (kind != KIND_SOLID) {
+                    // a warp of fluid and wall nodes pulls and sums once (a
+                    // wall node from its partner)
+                    const int d = kind == KIND_WALL ? partner_dir((uint8_t)c) : 0;
                     pull(lx + cx_rt(d), ly + cy_rt(d), g[j]);
                     moments<C>(g[j], dr[j], uu[j], vv[j]);
-                    const int sd = (c >> 20) & 7;
-                    nee<C>(g[j], dr[j], uu[j], vv[j], wall[2 * sd], wall[2 * sd + 1]);
+                    if (kind == KIND_WALL) {
+                        const int sd = (c >> 20) & 7;
+                        nee<C>(g[j], dr[j], uu[j], vv[j], wall[2 * sd], wall[2 * sd + 1]);
+                    }
                 } else {
                     uu[j] = vv[j] = C(0);
                 }
@@ -478,14 +479,13 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                 int lx, ly;
                 ring_node(tid - G::NT + j * G::RT, lx, ly);
                 C h[9], hd_, hu, hv;
-                if (ring_wall >> j & 1u) {
-                    const int d = partner_dir((uint8_t)rinfo[j]), sd = rinfo[j] >> 20;
-                    pull(lx + cx_rt(d), ly + cy_rt(d), h);
-                    moments<C>(h, hd_, hu, hv);
+                const bool w = ring_wall >> j & 1u;
+                const int d = w ? partner_dir((uint8_t)rinfo[j]) : 0;
+                pull(lx + cx_rt(d), ly + cy_rt(d), h);
+                moments<C>(h, hd_, hu, hv);
+                if (w) {
+                    const int sd = rinfo[j] >> 20;
                     nee<C>(h, hd_, hu, hv, wall[2 * sd], wall[2 * sd + 1]);
-                } else {
-                    pull(lx, ly, h);
-                    moments<C>(h, hd_, hu, hv);
                 }
                 RU[(ly + 1) * RW + lx + 1] = hu;
                 RV[(ly + 1) * RW + lx + 1] = hv;
