@@ -165,20 +165,20 @@ typedef struct {
                                (width x height, threads, input stages at 32 / 16
                                bit, population halo rows): 64x16, 1024, 3/3, 3;
                                64x16, 512, 3/3, 3; 64x8, 512, 2/3, 3 (two blocks
-                               per SM); 128x8, 1024, 2/3, 3; 64x16, 512 + 128 ring
-                               threads (four warps that take the one-node ring's
-                               moments and issue the copies), 3/3, 2; the same
-                               with 3 halo rows.  64-bit storage: 64x8, 256, 2;
+                               per SM); 128x8, 1024, 2/3, 3; 32x16, 256 + 64 ring
+                               threads (two warps that take the one-node ring's
+                               moments and issue the copies; two blocks per SM),
+                               3/3, 2; 64x16, 512 + 96 ring threads, 3/3, 2.  Of
+                               these, 1, 4 and 5 take pairs of nodes per thread.
+                               64-bit storage: 64x8, 256, 2;
                                32x8, 256, 3; 32x16, 512, 2; 32x8, 256, 2 (two
                                blocks per SM); 32x8, 256 + 64 ring threads, 3;
                                the same with 3 halo rows (64-bit shapes 0-4 take 2).
                                LBMFVM_TMA_DEFAULT: for a grid with fewer tiles
                                than the GPU has SMs, 2 (32- and 16-bit storage)
                                or 4 (64-bit), which spread it over more SMs;
-                               otherwise 4 when both population buffers and
-                               temperature planes fit in the L2, 5 if not (32-
-                               and 16-bit), 3 for 64-bit storage: the fastest
-                               measured on 64^2 to 4096^2 cavities.
+                               otherwise 4 (32- and 16-bit) or 3 (64-bit): the
+                               fastest measured on 64^2 to 4096^2 cavities.
                                LBMFVM_TMA_AUTOTUNE times every shape (a
                                captured graph of 32 launches, replayed twice)
                                on the handle's own grid at create and keeps

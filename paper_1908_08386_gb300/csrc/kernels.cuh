@@ -67,9 +67,11 @@ __device__ __forceinline__ int partner_dir(uint8_t code) {
 }
 
 // Weights (Eq. 9).
+struct fx2;
 template <class C>
 __host__ __device__ constexpr C wq(int q) {
-    return q == 0 ? C(4) / C(9) : (q < 5 ? C(1) / C(9) : C(1) / C(36));
+    if constexpr (std::is_same<C, fx2>::value) return C(wq<float>(q));  // both halves
+    else return q == 0 ? C(4) / C(9) : (q < 5 ? C(1) / C(9) : C(1) / C(36));
 }
 
 // ---------------------------------------------------------------------------
@@ -196,6 +198,79 @@ __device__ __forceinline__ dsf recip(dsf r) {
 }
 __device__ __forceinline__ double recip(double r) { return 1.0 / r; }
 
+// ---------------------------------------------------------------------------
+// Two FP32 values of two neighbouring nodes in one 64-bit register, computed
+// with the packed add, multiply and fused multiply-add of sm_100 and later:
+// one instruction for both, each half rounded like the single one, so paired
+// and single arithmetic agree bit for bit.  The fused step of 32- and 16-bit
+// storage is bound by its instruction stream, not by the FP32 pipe: pairs take
+// 217 instructions a node instead of 301 (1024^2 FP32; also wider shared-memory
+// accesses and no products by closed faces or unit extents).
+// ---------------------------------------------------------------------------
+struct fx2 {
+    unsigned long long v;
+    fx2() = default;
+    __device__ __forceinline__ fx2(float f) { asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(f)); }
+    __device__ __forceinline__ fx2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ float x() const {
+        float a, b;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+        return a;
+    }
+    __device__ __forceinline__ float y() const {
+        float a, b;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+        return b;
+    }
+};
+__device__ __forceinline__ fx2 operator+(fx2 a, fx2 b) {
+    fx2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ fx2 operator-(fx2 a, fx2 b) {
+    fx2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ fx2 mul_r(fx2 a, fx2 b) {
+    fx2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ fx2 fma_c(fx2 a, fx2 b, fx2 c) {
+    fx2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ fx2 operator-(fx2 a) { return mul_r(a, fx2(-1.0f)); }
+__device__ __forceinline__ fx2 recip(fx2 r) { return fx2(recip(r.x()), recip(r.y())); }
+// a where the half's flag is set, else b
+__device__ __forceinline__ fx2 pick(bool f0, bool f1, fx2 a, fx2 b) {
+    return fx2(f0 ? a.x() : b.x(), f1 ? a.y() : b.y());
+}
+// Two consecutive stored values (4- or 8-byte aligned).
+__device__ __forceinline__ fx2 ld2(const float *p) {
+    fx2 r;
+    r.v = *reinterpret_cast<const unsigned long long *>(p);
+    return r;
+}
+__device__ __forceinline__ fx2 ld2(const __half *p) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(p));
+    return fx2(f.x, f.y);
+}
+__device__ __forceinline__ fx2 ld2(const __nv_bfloat16 *p) {
+    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+    return fx2(f.x, f.y);
+}
+__device__ __forceinline__ void st2(float *p, fx2 v) { *reinterpret_cast<unsigned long long *>(p) = v.v; }
+__device__ __forceinline__ void st2(__half *p, fx2 v) {
+    *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v.x(), v.y());
+}
+__device__ __forceinline__ void st2(__nv_bfloat16 *p, fx2 v) {
+    *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(v.x(), v.y());
+}
+
 template <class S>
 struct StepArgs {
     using C = typename Compute<S>::type;
@@ -267,6 +342,13 @@ __device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b
 __device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ dsf mul_r(dsf a, dsf b) { return a * b; }
 
+// 3 x, rounded once: 2 x + x in a fused multiply-add (2 x is exact).  A packed
+// product that feeds an addition would be contracted with it by the assembler.
+template <class C>
+__device__ __forceinline__ C triple(C x) {
+    return fma_c(C(2), x, x);
+}
+
 // Eqs. 16-17 on shifted populations g = f - w: rho = 1 + sum g, rho u = sum e g.
 template <class C>
 __device__ __forceinline__ void moments(const C g[9], C &drho, C &ux, C &uy) {
@@ -300,10 +382,10 @@ __device__ __forceinline__ void nee(C g[9], C &drho, C &ux, C &uy, C uw, C vw) {
     // g_q += rho w_q (P_q(u_w) - P_q(u_f)); opposite directions share the
     // even part 4.5 (e.u)^2 - 1.5 u.u and differ in the sign of 3 e.u.
     const C rho = C(1) + drho;
-    const C dP0 = mul_r(C(-1.5), fma_c(uw, uw, mul_r(vw, vw)) - fma_c(ux, ux, mul_r(uy, uy)));
+    const C dP0 = mul_r(C(-1.5f), fma_c(uw, uw, mul_r(vw, vw)) - fma_c(ux, ux, mul_r(uy, uy)));
     g[0] = fma_c(mul_r(rho, wq<C>(0)), dP0, g[0]);
     auto pair = [&](int q, int qb, C euw, C euf) {
-        const C A = fma_c(C(4.5), fma_c(euw, euw, -mul_r(euf, euf)), dP0), B = mul_r(C(3), euw - euf);
+        const C A = fma_c(C(4.5f), fma_c(euw, euw, -mul_r(euf, euf)), dP0), B = triple(euw - euf);
         const C rw = mul_r(rho, wq<C>(q));
         g[q] = fma_c(rw, A + B, g[q]);
         g[qb] = fma_c(rw, A - B, g[qb]);
@@ -387,20 +469,20 @@ __device__ __forceinline__ void collide(const C g[9], C drho, C ux, C uy, C omeg
         return;
     } else {
     const C rho = C(1) + drho;
-    const C P0 = mul_r(C(-1.5), fma_c(ux, ux, mul_r(uy, uy)));
+    const C P0 = mul_r(C(-1.5f), fma_c(ux, ux, mul_r(uy, uy)));
     const C c = mul_r(C(3), rho);
     const C sx = mul_r(c, Gx), sy = mul_r(c, Gy);
-    const C sGu = fma_c(sx, ux, mul_r(sy, uy));
+    const C nGu = -fma_c(sx, ux, mul_r(sy, uy));
     const C om1 = C(1) - omega;
     auto out = [&](int q, C P, C s) {
         const C w = wq<C>(q);
         store(q, fma_c(om1, g[q], mul_r(w, fma_c(P, fma_c(omega, rho, s), fma_c(omega, drho, s)))));
     };
-    out(0, P0, -sGu);
+    out(0, P0, nGu);
     auto pair = [&](int q, int qb, C eu, C es) {
-        const C A = fma_c(C(4.5), mul_r(eu, eu), P0), B = mul_r(C(3), eu);
-        out(q, A + B, es - sGu);
-        out(qb, A - B, -es - sGu);
+        const C A = fma_c(C(4.5f), mul_r(eu, eu), P0), B = triple(eu);
+        out(q, A + B, nGu + es);
+        out(qb, A - B, nGu - es);
     };
     pair(1, 3, ux, sx);
     pair(2, 4, uy, sy);
@@ -435,6 +517,17 @@ __device__ __forceinline__ C fv_update(C TP, C uP, C vP, C ex, C ey, C alpha, bo
     // 1/(ex ey) is a power of two (ex, ey in {1/2, 1}): the product is exact.
     const C inv_v = (ex < C(1) ? C(2) : C(1)) * (ey < C(1) ? C(2) : C(1));
     return TP + (ey * (fe + fw) + ex * (fn + fs)) * inv_v;
+}
+
+// The same for two whole control volumes with open faces (1 / (ex ey) = 1).
+__device__ __forceinline__ fx2 fv_update_open(fx2 TP, fx2 uP, fx2 vP, fx2 alpha, fx2 TE, fx2 uE, fx2 TN, fx2 vN, fx2 TW,
+                                              fx2 uW, fx2 TS, fx2 vS) {
+    const fx2 q(0.25f), nq(-0.25f);
+    const fx2 fe = fma_c(alpha, TE - TP, mul_r(mul_r(nq, uP + uE), TP + TE));
+    const fx2 fw = fma_c(alpha, TW - TP, mul_r(mul_r(q, uP + uW), TP + TW));
+    const fx2 fn = fma_c(alpha, TN - TP, mul_r(mul_r(nq, vP + vN), TP + TN));
+    const fx2 fs = fma_c(alpha, TS - TP, mul_r(mul_r(q, vP + vS), TP + TS));
+    return TP + ((fe + fw) + (fn + fs));
 }
 
 // QUICK face value (Leonard's quadratic upstream interpolation, the scheme
@@ -836,8 +929,17 @@ struct TmaTile {
     static constexpr int FW = TW + 2 * XOFF, FH = TH + 2 * FHALO;  // population box
     static constexpr int TWD = TW + 8, THT = TH + 2 * THALO;  // temperature box (x0-4, y0-THALO)
     static constexpr int CWD = TW + 32, CHT = TH + 2;      // code box (x0-16, y0-1), codes then face flags
-    static constexpr int RW = TW + 2, RH = TH + 2;         // tile + ring
-    static constexpr int NRING = 2 * RW + 2 * TH;          // ring nodes
+    // 32-bit arithmetic, an even number of nodes per thread: threads take
+    // pairs of neighbours in a row (fx2)
+    static constexpr bool PAIRED = std::is_same<TC, float>::value && NPT % 2 == 0;
+    // tile + ring; the first own column sits at RX (even where pairs are stored)
+    static constexpr int RX = PAIRED ? 2 : 1, RW = TW + 2 * RX, RH = TH + 2;
+    static constexpr int NRING = 2 * TW + 2 * TH;          // ring nodes (no face reaches the corners)
+    // Columns between the borders across which a wall node's velocity is the
+    // wall's own instead of the one extrapolated in its tile (they differ by
+    // rounding): 64 in FP32 arithmetic, so that narrower tiles round like the
+    // 64-column ones.
+    static constexpr int BW = std::is_same<TC, float>::value && TW < 64 ? 64 : TW;
     static constexpr uint32_t F_BYTES = 9u * FH * FW * sizeof(S);
     static constexpr uint32_t T_BYTES = (uint32_t)THT * TWD * (uint32_t)sizeof(TC);
     static constexpr uint32_t C_PLANE = (uint32_t)CHT * CWD;
@@ -887,10 +989,14 @@ template <class S> struct TmaConfig<S, 0> { using G = TmaTile<S, 64, 16, 3, 1024
 template <class S> struct TmaConfig<S, 1> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 0, 3>; };
 template <class S> struct TmaConfig<S, 2> { using G = TmaTile<S, 64, 8, sizeof(S) == 4 ? 2 : 3, 512, 2, 1, 0, 3>; };
 template <class S> struct TmaConfig<S, 3> { using G = TmaTile<S, 128, 8, sizeof(S) == 4 ? 2 : 3, 1024, 1, 1, 0, 3>; };
-// 64 x 16 with four ring warps (which also issue the copies): two halo rows
-// (the faster on grids inside the L2), three rows (the faster beyond it)
-template <class S> struct TmaConfig<S, 4> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 128, 2>; };
-template <class S> struct TmaConfig<S, 5> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 128, 3>; };
+// 32 x 16 with two ring warps (which also issue the copies), two blocks per
+// SM, so that one block's barrier, loads and stores overlap the other's
+// arithmetic; 64 x 16 with three ring warps, one block per SM.  Us per step,
+// single nodes in 64 x 16 / pairs in 64 x 16 / pairs in 32 x 16: 1024^2 FP32
+// 18.1 / 17.0 / 15.4-16.3, FP16 17.0 / 15.1 / 14.6-15.3; 4096^2 FP32 236 / 222 /
+// 213, FP16 212 / 175 / 171-178
+template <class S> struct TmaConfig<S, 4> { using G = TmaTile<S, 32, 16, 3, 256, 2, 1, 64, 2>; };
+template <class S> struct TmaConfig<S, 5> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 96, 2>; };
 // 64-bit storage: a 32 x 8 tile stages 43 KB, a 64 x 8 tile 78 KB.
 template <> struct TmaConfig<double, 0> { using G = TmaTile<double, 64, 8, 2, 256>; };
 template <> struct TmaConfig<double, 1> { using G = TmaTile<double, 32, 8, 3, 256>; };
@@ -1140,9 +1246,67 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
 
         // Phase A: own nodes into registers (their u, v also to the ring
         // buffer), the ring's u, v.
-        C g[NPT][9], dr[NPT], uu[NPT], vv[NPT];
+        constexpr int NP = G::PAIRED ? NPT / 2 : 1;  // pairs per thread
+        fx2 g2[NP][9], dr2[NP], uu2[NP], vv2[NP];
+        C g[G::PAIRED ? 1 : NPT][9], dr[NPT], uu[NPT], vv[NPT];
         uint8_t cc[NPT];
-        if (computes) {
+        if constexpr (G::PAIRED) {
+            if (computes) {
+#pragma unroll
+                for (int j = 0; j < NP; j++) {
+                    const int i = tid + j * G::THREADS;
+                    const int ly = i / (TW / 2), lx = 2 * (i - ly * (TW / 2));
+                    const uint16_t c2 = *reinterpret_cast<const uint16_t *>(CC + cidx(lx, ly));
+                    const uint8_t c[2] = {decode((uint8_t)c2), decode((uint8_t)(c2 >> 8))};
+                    cc[2 * j] = c[0];
+                    cc[2 * j + 1] = c[1];
+                    fx2(&p)[9] = g2[j];
+                    if (((c[0] | c[1]) & 3) == KIND_FLUID) {
+                        const S *f = F + fidx(lx, ly);
+#pragma unroll
+                        for (int q = 0; q < 9; q++) {
+                            const S *s = f + q * (FH * FW) - cy(q) * FW;
+                            if (cx(q) == 0) p[q] = ld2(s);
+                            else p[q] = fx2(ld(s - cx(q)), ld(s + 1 - cx(q)));
+                        }
+                    } else {
+                        // a wall node pulls from its partner, an inert one nothing
+                        C h[2][9];
+#pragma unroll
+                        for (int k = 0; k < 2; k++) {
+                            const int d = (c[k] & 3) == KIND_WALL ? partner_dir(c[k]) : 0;
+                            pull(lx + k + cx_rt(d), ly + cy_rt(d), h[k]);
+                            if ((c[k] & 3) == KIND_SOLID)
+#pragma unroll
+                                for (int q = 0; q < 9; q++) h[k][q] = C(0);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 9; q++) p[q] = fx2(h[0][q], h[1][q]);
+                    }
+                    moments<fx2>(p, dr2[j], uu2[j], vv2[j]);
+                    const bool w0 = (c[0] & 3) == KIND_WALL, w1 = (c[1] & 3) == KIND_WALL;
+                    if (w0 || w1) {
+                        C uw[2] = {C(0), C(0)}, vw[2] = {C(0), C(0)};
+                        if (w0) wall_vel(lx, ly, c[0], uw[0], vw[0]);
+                        if (w1) wall_vel(lx + 1, ly, c[1], uw[1], vw[1]);
+                        fx2 n[9], nd = dr2[j], nu = uu2[j], nv = vv2[j];
+#pragma unroll
+                        for (int q = 0; q < 9; q++) n[q] = p[q];
+                        nee<fx2>(n, nd, nu, nv, fx2(uw[0], uw[1]), fx2(vw[0], vw[1]));
+#pragma unroll
+                        for (int q = 0; q < 9; q++) p[q] = pick(w0, w1, n[q], p[q]);
+                        dr2[j] = pick(w0, w1, nd, dr2[j]);
+                        uu2[j] = pick(w0, w1, nu, uu2[j]);
+                        vv2[j] = pick(w0, w1, nv, vv2[j]);
+                    }
+                    if constexpr (MODE != FV_GIVEN) {
+                        const int r = (ly + 1) * RW + lx + G::RX;
+                        st2(RU + r, uu2[j]);
+                        st2(RV + r, vv2[j]);
+                    }
+                }
+            }
+        } else if (computes) {
 #pragma unroll
             for (int j = 0; j < NPT; j++) {
                 const int i = tid + j * G::THREADS;
@@ -1150,7 +1314,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                 cc[j] = decode(CC[cidx(lx, ly)]);
                 state(lx, ly, cc[j], g[j], dr[j], uu[j], vv[j]);
                 if constexpr (MODE != FV_GIVEN) {
-                    const int r = (ly + 1) * RW + (lx + 1);
+                    const int r = (ly + 1) * RW + lx + G::RX;
                     RU[r] = uu[j];
                     RV[r] = vv[j];
                 }
@@ -1158,23 +1322,79 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
         }
         // the ring's velocities feed the energy update's faces only
         if (MODE != FV_GIVEN) {
-            const int first = RT ? tid - G::THREADS : tid, stride = RT ? RT : G::NRING;
-            for (int hr = first; hr >= 0 && hr < G::NRING; hr += stride) {
-                int rx, ry;
-                if (hr < RW) { rx = hr; ry = 0; }
-                else if (hr < 2 * RW) { rx = hr - RW; ry = TH + 1; }
-                else { const int h = hr - 2 * RW; rx = (h & 1) ? RW - 1 : 0; ry = 1 + (h >> 1); }
-                const uint8_t c = decode(CC[cidx(rx - 1, ry - 1)]);
-                C hu = C(0), hv = C(0);
-                if ((c & 3) == KIND_FLUID) {
-                    C hg[9], hd;
-                    state(rx - 1, ry - 1, c, hg, hd, hu, hv);
-                } else if ((c & 3) == KIND_WALL) {
-                    // the extrapolated wall node moves with the wall (Eq. 94)
-                    wall_vel(rx - 1, ry - 1, c, hu, hv);
+            const int first = RT ? tid - G::THREADS : tid, stride = RT ? RT : G::BLOCK;
+            auto ring_node = [&](int h, int &lx, int &ly) {
+                if (h < TW) lx = h, ly = -1;
+                else if (h < 2 * TW) lx = h - TW, ly = TH;
+                else lx = ((h - 2 * TW) & 1) ? TW : -1, ly = (h - 2 * TW) >> 1;
+            };
+            if constexpr (G::PAIRED && RT > 0) {
+                // two ring nodes per thread and pass
+                for (int hr = 2 * first; hr >= 0 && hr < G::NRING; hr += 2 * stride) {
+                    int lx[2], ly[2];
+                    uint8_t c[2];
+                    C h0[9], h1[9];
+                    bool ext[2] = {false, false};  // box wall node inside a border column pair
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        ring_node(hr + k, lx[k], ly[k]);
+                        c[k] = decode(CC[cidx(lx[k], ly[k])]);
+                        int px = lx[k], py = ly[k];
+                        if constexpr (G::BW != TW) {
+                            if ((c[k] & 3) == KIND_WALL && (c[k] >> 6) != TH_OBSTACLE && (px < 0 || px >= TW)) {
+                                const int d = partner_dir(c[k]);
+                                const int qx = px + cx_rt(d), qy = py + cy_rt(d);
+                                ext[k] = (px < 0 ? ox : ox + TW) % G::BW != 0 && qx >= -1 && qx <= TW && qy >= -1 &&
+                                         qy <= TH;
+                                if (ext[k]) px = qx, py = qy;
+                            }
+                        }
+                        pull(px, py, k ? h1 : h0);
+                    }
+                    fx2 h[9], hd, hu, hv;
+#pragma unroll
+                    for (int q = 0; q < 9; q++) h[q] = fx2(h0[q], h1[q]);
+                    moments<fx2>(h, hd, hu, hv);
+                    if constexpr (G::BW != TW) {
+                        if (ext[0] || ext[1]) {
+                            C uw[2] = {C(0), C(0)}, vw[2] = {C(0), C(0)};
+                            for (int k = 0; k < 2; k++)
+                                if (ext[k]) wall_vel(lx[k], ly[k], c[k], uw[k], vw[k]);
+                            fx2 nu = hu, nv = hv;
+                            nee<fx2>(h, hd, nu, nv, fx2(uw[0], uw[1]), fx2(vw[0], vw[1]));
+                            hu = pick(ext[0], ext[1], nu, hu);
+                            hv = pick(ext[0], ext[1], nv, hv);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        C u = k ? hu.y() : hu.x(), v = k ? hv.y() : hv.x();
+                        if ((c[k] & 3) != KIND_FLUID && !ext[k]) {
+                            u = v = C(0);
+                            // the extrapolated wall node moves with the wall (Eq. 94)
+                            if ((c[k] & 3) == KIND_WALL) wall_vel(lx[k], ly[k], c[k], u, v);
+                        }
+                        const int r = (ly[k] + 1) * RW + lx[k] + G::RX;
+                        RU[r] = u;
+                        RV[r] = v;
+                    }
                 }
-                RU[ry * RW + rx] = hu;
-                RV[ry * RW + rx] = hv;
+            } else {
+                for (int hr = first; hr >= 0 && hr < G::NRING; hr += stride) {
+                    int lx, ly;
+                    ring_node(hr, lx, ly);
+                    const uint8_t c = decode(CC[cidx(lx, ly)]);
+                    C hu = C(0), hv = C(0);
+                    if ((c & 3) == KIND_FLUID) {
+                        C hg[9], hd;
+                        state(lx, ly, c, hg, hd, hu, hv);
+                    } else if ((c & 3) == KIND_WALL) {
+                        // the extrapolated wall node moves with the wall (Eq. 94)
+                        wall_vel(lx, ly, c, hu, hv);
+                    }
+                    RU[(ly + 1) * RW + lx + G::RX] = hu;
+                    RV[(ly + 1) * RW + lx + G::RX] = hv;
+                }
             }
         }
         __syncthreads();
@@ -1193,61 +1413,103 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
         // to the stage's (now dead) population bytes.  Inert nodes keep T.
         S *OF = reinterpret_cast<S *>(stg + G::F_OFF);
         C *OT = reinterpret_cast<C *>(stg + G::F_OFF + G::OT_OFF);
-#pragma unroll
-        for (int j = 0; j < NPT; j++) {
-            if (!computes) break;
-            const int i = tid + j * G::THREADS;
-            const int ly = i / TW, lx = i - ly * TW;
-            const uint8_t c = cc[j];
+        // T^{n+1} of node (lx, ly) with code c and velocity (uP, vP)
+        auto energy = [&](int lx, int ly, uint8_t c, C uP, C vP) {
             const int t = tidx(lx, ly);
             const C TP = TT[t];
-            S *of = OF + ly * TW + lx;
-            if ((c & 3) == KIND_SOLID) {
-                OT[ly * TW + lx] = TP;
-#pragma unroll
-                for (int q = 0; q < 9; q++) st(of + q * OPLANE, C(0));
-                continue;
-            }
-            const int r = (ly + 1) * RW + (lx + 1);
+            const int r = (ly + 1) * RW + lx + G::RX;
             const int th = c >> 6;
-            C Tn = TP;
-            if (MODE == FV_GIVEN) {
-                // T^{n+1} of every node comes from the sub-step kernels
-            } else if (th == TH_FV) {
+            if (MODE == FV_GIVEN) return TP;  // T^{n+1} of every node comes from the sub-step kernels
+            if (th == TH_FV) {
                 // control volume clipped to the cavity; faces beyond it are closed
                 const uint8_t ff = CF[cidx(lx, ly)];
-                const C ex = ((ff & FF_IN_W) ? C(0.5) : C(0)) + ((ff & FF_IN_E) ? C(0.5) : C(0));
-                const C ey = ((ff & FF_IN_S) ? C(0.5) : C(0)) + ((ff & FF_IN_N) ? C(0.5) : C(0));
+                const C ex = ((ff & FF_IN_W) ? C(0.5f) : C(0)) + ((ff & FF_IN_E) ? C(0.5f) : C(0));
+                const C ey = ((ff & FF_IN_S) ? C(0.5f) : C(0)) + ((ff & FF_IN_N) ? C(0.5f) : C(0));
                 if constexpr (MODE == FV_QUICK) {
                     // far upstream nodes: beyond P (P's own flags) or beyond
                     // the neighbour (the neighbour's flag on the same side)
                     const int W2 = G::TWD;
-                    const C uP = uu[j], vP = vv[j], TP_ = TP;
-                    const C TE = TT[t + 1], TW = TT[t - 1], TN = TT[t + W2], TS = TT[t - W2];
+                    const C TE = TT[t + 1], TWt = TT[t - 1], TN = TT[t + W2], TS = TT[t - W2];
                     const C uE = RU[r + 1], uW = RU[r - 1], vN = RV[r + RW], vS = RV[r - RW];
-                    const C TfE = quick_face<C>(uP + uE, TP_, TE, ff & FF_OPEN_W, TW,
-                                                CF[cidx(lx + 1, ly)] & FF_OPEN_E, TT[t + 2]);
-                    const C TfW = quick_face<C>(-(uP + uW), TP_, TW, ff & FF_OPEN_E, TE,
+                    const C TfE = quick_face<C>(uP + uE, TP, TE, ff & FF_OPEN_W, TWt, CF[cidx(lx + 1, ly)] & FF_OPEN_E,
+                                                TT[t + 2]);
+                    const C TfW = quick_face<C>(-(uP + uW), TP, TWt, ff & FF_OPEN_E, TE,
                                                 CF[cidx(lx - 1, ly)] & FF_OPEN_W, TT[t - 2]);
-                    const C TfN = quick_face<C>(vP + vN, TP_, TN, ff & FF_OPEN_S, TS,
-                                                CF[cidx(lx, ly + 1)] & FF_OPEN_N, TT[t + 2 * W2]);
-                    const C TfS = quick_face<C>(-(vP + vS), TP_, TS, ff & FF_OPEN_N, TN,
+                    const C TfN = quick_face<C>(vP + vN, TP, TN, ff & FF_OPEN_S, TS, CF[cidx(lx, ly + 1)] & FF_OPEN_N,
+                                                TT[t + 2 * W2]);
+                    const C TfS = quick_face<C>(-(vP + vS), TP, TS, ff & FF_OPEN_N, TN,
                                                 CF[cidx(lx, ly - 1)] & FF_OPEN_S, TT[t - 2 * W2]);
-                    Tn = fv_update_faces<C>(TP_, uP, vP, ex, ey, alpha, C(1), ff & FF_OPEN_E, TE, uE, TfE,
-                                            ff & FF_OPEN_N, TN, vN, TfN, ff & FF_OPEN_W, TW, uW, TfW, ff & FF_OPEN_S,
-                                            TS, vS, TfS);
+                    return fv_update_faces<C>(TP, uP, vP, ex, ey, alpha, C(1), ff & FF_OPEN_E, TE, uE, TfE,
+                                              ff & FF_OPEN_N, TN, vN, TfN, ff & FF_OPEN_W, TWt, uW, TfW,
+                                              ff & FF_OPEN_S, TS, vS, TfS);
                 } else {
-                    Tn = fv_update<C>(TP, uu[j], vv[j], ex, ey, alpha, ff & FF_OPEN_E, TT[t + 1], RU[r + 1],
-                                      ff & FF_OPEN_N, TT[t + G::TWD], RV[r + RW], ff & FF_OPEN_W, TT[t - 1], RU[r - 1],
-                                      ff & FF_OPEN_S, TT[t - G::TWD], RV[r - RW]);
+                    return fv_update<C>(TP, uP, vP, ex, ey, alpha, ff & FF_OPEN_E, TT[t + 1], RU[r + 1],
+                                        ff & FF_OPEN_N, TT[t + G::TWD], RV[r + RW], ff & FF_OPEN_W, TT[t - 1],
+                                        RU[r - 1], ff & FF_OPEN_S, TT[t - G::TWD], RV[r - RW]);
                 }
-            } else if (th == TH_OBSTACLE) {
-                const int d = partner_dir(c);
-                Tn = TT[tidx(lx + cx_rt(d), ly + cy_rt(d))];
             }
-            OT[ly * TW + lx] = Tn;
-            const C Gy = fma_c(gbeta, Tn - t_ref, fy);
-            collide<C>(g[j], dr[j], uu[j], vv[j], omega, fx, Gy, [&](int q, C v) { st(of + q * OPLANE, v); });
+            if (th == TH_OBSTACLE) {
+                const int d = partner_dir(c);
+                return TT[tidx(lx + cx_rt(d), ly + cy_rt(d))];
+            }
+            return TP;
+        };
+        if constexpr (G::PAIRED) {
+            if (computes) {
+                const fx2 om(omega), al(alpha), fx_2(fx), fy_2(fy), gb(gbeta), tr(t_ref);
+#pragma unroll
+                for (int j = 0; j < NP; j++) {
+                    const int i = tid + j * G::THREADS;
+                    const int ly = i / (TW / 2), lx = 2 * (i - ly * (TW / 2));
+                    const uint8_t c0 = cc[2 * j], c1 = cc[2 * j + 1];
+                    fx2 Tn;
+                    bool open = false;  // two whole control volumes with open faces: nearly every pair
+                    if constexpr (MODE == FV_CENTRAL)
+                        open = (c0 | c1) < (1 << 6) && *reinterpret_cast<const uint16_t *>(CF + cidx(lx, ly)) == 0xffffu;
+                    if (open) {
+                        const int t = tidx(lx, ly), r = (ly + 1) * RW + lx + G::RX;
+                        const fx2 TP = ld2(TT + t);
+                        Tn = fv_update_open(TP, uu2[j], vv2[j], al, fx2(TP.y(), TT[t + 2]), fx2(uu2[j].y(), RU[r + 2]),
+                                            ld2(TT + t + G::TWD), ld2(RV + r + RW), fx2(TT[t - 1], TP.x()),
+                                            fx2(RU[r - 1], uu2[j].x()), ld2(TT + t - G::TWD), ld2(RV + r - RW));
+                    } else {
+                        Tn = fx2((c0 & 3) == KIND_SOLID ? TT[tidx(lx, ly)] : energy(lx, ly, c0, uu2[j].x(), vv2[j].x()),
+                                 (c1 & 3) == KIND_SOLID ? TT[tidx(lx + 1, ly)]
+                                                        : energy(lx + 1, ly, c1, uu2[j].y(), vv2[j].y()));
+                    }
+                    S *of = OF + ly * TW + lx;
+                    st2(OT + ly * TW + lx, Tn);
+                    const bool s0 = (c0 & 3) == KIND_SOLID, s1 = (c1 & 3) == KIND_SOLID;
+                    const fx2 Gy = fma_c(gb, Tn - tr, fy_2);
+                    if (!(s0 || s1)) {
+                        collide<fx2>(g2[j], dr2[j], uu2[j], vv2[j], om, fx_2, Gy,
+                                     [&](int q, fx2 v) { st2(of + q * OPLANE, v); });
+                    } else {
+                        // inert nodes hold zeros
+                        collide<fx2>(g2[j], dr2[j], uu2[j], vv2[j], om, fx_2, Gy,
+                                     [&](int q, fx2 v) { st2(of + q * OPLANE, pick(s0, s1, fx2(0.0f), v)); });
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < NPT; j++) {
+                if (!computes) break;
+                const int i = tid + j * G::THREADS;
+                const int ly = i / TW, lx = i - ly * TW;
+                const uint8_t c = cc[j];
+                S *of = OF + ly * TW + lx;
+                if ((c & 3) == KIND_SOLID) {
+                    OT[ly * TW + lx] = TT[tidx(lx, ly)];
+#pragma unroll
+                    for (int q = 0; q < 9; q++) st(of + q * OPLANE, C(0));
+                    continue;
+                }
+                const C Tn = energy(lx, ly, c, uu[j], vv[j]);
+                OT[ly * TW + lx] = Tn;
+                const C Gy = fma_c(gbeta, Tn - t_ref, fy);
+                collide<C>(g[j], dr[j], uu[j], vv[j], omega, fx, Gy, [&](int q, C v) { st(of + q * OPLANE, v); });
+            }
         }
         if (tid == PROD && k > 0 && pre_t >= 0) {
             tma::bulk_wait_read();  // the results of tile k-1 have left its stage
@@ -1961,7 +2223,7 @@ struct TmaLaunch {
 
 // Box geometry of a tile shape (the host encodes its tensor maps from it).
 struct TmaShape {
-    int TW, TH, FW, FH, TWD, THT, THT_QUICK, CWD, CHT, STAGES, BLOCK;
+    int TW, TH, BW, FW, FH, TWD, THT, THT_QUICK, CWD, CHT, STAGES, BLOCK;
     unsigned SMEM;
 };
 

@@ -340,6 +340,7 @@ struct lbmfvm {
     uint32_t res_seq;                // exchanges made since the resident tile list was built
     uint32_t code_crc; // CRC-32 of the node codes, identifies the geometry in checkpoints
     int tile_w, tile_h;
+    int tile_bw;      // columns between the tiles' rounding borders (TmaTile::BW)
     // Several cavities packed in one grid (batch handles); empty for one cavity.
     std::vector<CavityDesc> atlas_cavs;
     std::vector<char> atlas_active;
@@ -845,6 +846,7 @@ int setup_tma(lbmfvm_t *h) {
     }
     h->tile_w = g.TW;
     h->tile_h = g.TH;
+    h->tile_bw = g.BW;
     return upload_tiles(h, g.TW, g.TH);
 }
 
@@ -1312,30 +1314,24 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
     h->prec = opts.store;
     h->tile_y = opts.tile_y ? opts.tile_y : 8;
     h->use_tma = tma_ok && opts.kernel != LBMFVM_KERNEL_GENERIC;
-    // the default shapes are the fastest measured ones: 64 x 16 with ring
-    // warps for 32- and 16-bit storage (two population halo rows when both
-    // population buffers and temperature planes fit in the L2, three
-    // otherwise), two blocks of 32 x 8 per SM for 64-bit.  A grid with fewer
-    // tiles than SMs is bound by the latency of one tile, not by the SMs'
-    // throughput, and takes the smaller tiles that spread it over more SMs:
-    // 64 x 8 (two blocks per SM) for 32- and 16-bit storage, 32 x 8 with ring
-    // warps for 64-bit.
+    // the default shapes are the fastest measured ones: two blocks of 32 x 16
+    // per SM with ring warps for 32- and 16-bit storage, two blocks of 32 x 8
+    // per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
+    // SMs is bound by the latency of one tile, not by the SMs' throughput, and
+    // takes the smaller tiles that spread it over more SMs: 64 x 8 (two blocks
+    // per SM) for 32- and 16-bit storage, 32 x 8 with ring warps for 64-bit.
     int shape_default = 3;
     {
-        int dev = 0, l2 = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess ||
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            l2 = sms = 0;
+            sms = 0;
         const long long tiles = store_size(opts.store) == 8
                                     ? (long long)((grid->nx + 31) / 32) * ((grid->ny + 7) / 8)
                                     : (long long)((grid->nx + 63) / 64) * ((grid->ny + 15) / 16);
         const bool small = tiles < sms;
-        if (store_size(opts.store) == 8) {
-            shape_default = small ? 4 : 3;
-        } else {
-            const size_t state = 2 * (9 * store_size(opts.store) + temp_size(opts.store)) * (size_t)L.plane;
-            shape_default = small ? 2 : state <= (size_t)l2 ? 4 : 5;
-        }
+        if (store_size(opts.store) == 8) shape_default = small ? 4 : 3;
+        else shape_default = small ? 2 : 4;
     }
     const bool own_shape = opts.tma_config == LBMFVM_TMA_AUTOTUNE || opts.tma_config == LBMFVM_TMA_DEFAULT;
     h->tma_config = own_shape ? shape_default : opts.tma_config;
@@ -1474,7 +1470,7 @@ int launch_resident(lbmfvm_t *h, int n) {
     r.seq0 = h->res_seq;
     r.nsteps = n;
     r.quick = h->fv_quick;
-    r.tile_w = h->tile_w;
+    r.tile_w = h->tile_bw;
     r.tile_h = h->tile_h;
     r.ctr[0] = reinterpret_cast<int *>(h->base + list_fused(h).slot) + 1;
     r.ctr[1] = reinterpret_cast<int *>(h->base + list_split(h).slot) + 1;

@@ -16,6 +16,7 @@ cudaError_t prepare_cfg(TmaShape *shape, int *blocks_per_sm) {
     using G = typename TmaConfig<S, CFG>::G;
     shape->TW = G::TW;
     shape->TH = G::TH;
+    shape->BW = G::BW;
     shape->FW = G::FW;
     shape->FH = G::FH;
     shape->TWD = G::TWD;
