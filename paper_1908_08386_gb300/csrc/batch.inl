@@ -144,7 +144,8 @@ void launch_cav_residual(lbmfvm_batch_t *b, int i, int update_only) {
     residual_kernel<S><<<blocks, 256, 0, h->s>>>(v, direct, su, sv, red, update_only);
     if (!update_only)
         residual_finish_kernel<<<1, 32, 0, h->s>>>(red, blocks,
-                                                   reinterpret_cast<double *>(h->base + h->L.cavres) + kCavRes * i);
+                                                   reinterpret_cast<double *>(h->base + h->L.cavres) + kCavRes * i, v.err,
+                                                   nullptr);
 }
 
 template <class S>
@@ -156,7 +157,8 @@ void launch_cav_nusselt(lbmfvm_batch_t *b, int i) {
     double *red = reinterpret_cast<double *>(h->base + h->L.red);
     nusselt_kernel<S><<<1, 256, 0, h->s>>>(v, (double)(g.ny - 1), g.t_wall[LBMFVM_SIDE_W] - g.t_wall[LBMFVM_SIDE_E],
                                            red + kRedLocal,
-                                           reinterpret_cast<double *>(h->base + h->L.cavres) + kCavRes * i + kCavNu);
+                                           reinterpret_cast<double *>(h->base + h->L.cavres) + kCavRes * i + kCavNu,
+                                           nullptr);
 }
 
 template <class S>
@@ -172,12 +174,13 @@ void launch_cav_rescale(lbmfvm_batch_t *b, int i) {
     rescale_kernel<S><<<grid, block, 0, h->s>>>(v, f0, f1, tot);
 }
 
-template <class S, class O>
-void launch_cav_fields(lbmfvm_batch_t *b, int i, int which, O *o0, O *o1) {
+template <class S>
+void launch_cav_fields(lbmfvm_batch_t *b, int i, double *const *o) {
     int direct;
     StepArgs<S> v = cav_read_view<S>(b, i, direct);
     dim3 block(32, 8), grid((v.nx + 31) / 32, (v.ny + 7) / 8);
-    fields_kernel<S, O><<<grid, block, 0, hnd(b, i)->s>>>(v, direct, which, o0, o1);
+    fields_kernel<S, double><<<grid, block, 0, hnd(b, i)->s>>>(v, direct, o[0], o[1], o[2], o[3],
+                                                               hnd(b, i)->host + kHostStatus);
 }
 
 // FN<storage type>(...) for the precision of packed grid h.
@@ -642,26 +645,12 @@ int lbmfvm_batch_fields(lbmfvm_batch_t *b, int32_t i, double *rho, double *u, do
     if (int r = check_index(b, i)) return r;
     lbmfvm_t *h = hnd(b, i);
     const size_t n = (size_t)b->cav[i].grid.nx * b->cav[i].grid.ny;
-    double *st = reinterpret_cast<double *>(h->base + h->L.stage);
     if (int r = bcheck_h(b, h, join_in(h))) return r;
-    double *outs[2][2] = {{rho, u}, {v, T}};
-    cudaError_t e = cudaSuccess;
-    for (int which = 0; which < 2 && e == cudaSuccess; which++) {
-        if (!outs[which][0] && !outs[which][1]) continue;
-        switch (h->prec) {
-            case LBMFVM_F64: launch_cav_fields<double, double>(b, i, which, st, st + n); break;
-            case LBMFVM_F32: launch_cav_fields<float, double>(b, i, which, st, st + n); break;
-            case LBMFVM_F16: launch_cav_fields<__half, double>(b, i, which, st, st + n); break;
-            case LBMFVM_BF16: launch_cav_fields<__nv_bfloat16, double>(b, i, which, st, st + n); break;
-            case LBMFVM_F32X2: launch_cav_fields<dsf, double>(b, i, which, st, st + n); break;
-        }
-        e = cudaGetLastError();
-        for (int k = 0; k < 2 && e == cudaSuccess; k++)
-            if (outs[which][k]) e = cudaMemcpyAsync(outs[which][k], st + k * n, n * sizeof(double), cudaMemcpyDefault, h->s);
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
+    double *const outs[4] = {rho, u, v, T};
+    cudaError_t e = copy_fields<double>(h, n, outs, [&](double *const *o) { BDISPATCH(h, launch_cav_fields, b, i, o); });
+    if (e == cudaSuccess && !rho && !u && !v && !T) e = cudaStreamSynchronize(h->s);
     if (e != cudaSuccess) return bfail(b, LBMFVM_ERR_CUDA, "batch fields failed: %s", cudaGetErrorString(e));
-    if (int r = bcheck_h(b, h, check_device_status(h))) return r;
+    if (int r = bcheck_h(b, h, rho || u || v || T ? wait_results(h) : check_device_status(h))) return r;
     return bcheck_h(b, h, join_out(h));
 }
 

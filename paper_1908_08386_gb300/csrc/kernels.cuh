@@ -2045,27 +2045,27 @@ __device__ __forceinline__ void current_moments(const StepArgs<S> &a, int direct
     }
 }
 
-// Field export: two of (rho, u, v, T) selected by `which` (0 = rho,u; 1 = v,T)
-// into out0/out1 (row-major ny*nx), in double or float.
+// Field export of rho, u, v, T (those that are not NULL; row-major ny*nx), in
+// double or float: one pull per node for all of them.  status (may be NULL,
+// host-mapped) receives the device status word.
 template <class S, class O>
-__global__ void fields_kernel(const StepArgs<S> a, int direct, int which, O *out0, O *out1) {
+__global__ void fields_kernel(const StepArgs<S> a, int direct, O *rho, O *u, O *v, O *T, double *status) {
     using C = typename Compute<S>::type;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x == 0 && y == 0 && status) *status = (double)*a.err;
     if (x >= a.nx || y >= a.ny) return;
     const long long k = (long long)y * a.pitch + x;
     const long long ko = (long long)y * a.nx + x;
-    const uint8_t c = decode(a.code[k]);
-    C drho, ux, uy;
-    current_moments<S>(a, direct, x, y, c, drho, ux, uy);
-    const bool inert = (c & 3) == KIND_SOLID;
-    if (which == 0) {
-        out0[ko] = O(inert ? C(0) : C(1) + drho);
-        out1[ko] = O(ux);
-    } else {
-        out0[ko] = O(uy);
-        out1[ko] = O(a.Tin[k]);
+    if (rho || u || v) {
+        const uint8_t c = decode(a.code[k]);
+        C drho, ux, uy;
+        current_moments<S>(a, direct, x, y, c, drho, ux, uy);
+        if (rho) rho[ko] = O((c & 3) == KIND_SOLID ? C(0) : C(1) + drho);
+        if (u) u[ko] = O(ux);
+        if (v) v[ko] = O(uy);
     }
+    if (T) T[ko] = O(a.Tin[k]);
 }
 
 // Residual, pass 1: per-block FP64 sums of |u - u_snap|^2 and |u|^2 over
@@ -2075,6 +2075,9 @@ __global__ void fields_kernel(const StepArgs<S> a, int direct, int which, O *out
 // Sums of the residual pass, per block and in total: |u - u_s|^2, |u|^2,
 // rho - 1 and the node count, all over the fluid nodes.
 constexpr int kResidualSums = 4;
+// Host-mapped results of a handle: sums or means, the device status word, and
+// from kHostLocal the local Nusselt numbers.
+constexpr int kHostStatus = 8, kHostLocal = 16;
 
 template <class S>
 __global__ void __launch_bounds__(256) residual_kernel(const StepArgs<S> a, int direct, double *su,
@@ -2116,8 +2119,10 @@ __global__ void __launch_bounds__(256) residual_kernel(const StepArgs<S> a, int 
     }
 }
 
-// Residual, pass 2: one warp sums the block partials in a fixed order.
-static __global__ void residual_finish_kernel(const double *partials, int nblocks, double *out) {
+// Residual, pass 2: one warp sums the block partials in a fixed order.  host
+// (may be NULL, host-mapped) receives the totals and the device status word.
+static __global__ void residual_finish_kernel(const double *partials, int nblocks, double *out, const int *err,
+                                              double *host) {
     double v[kResidualSums] = {};
     for (int b = threadIdx.x; b < nblocks; b += 32)
 #pragma unroll
@@ -2127,9 +2132,14 @@ static __global__ void residual_finish_kernel(const double *partials, int nblock
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
     }
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
 #pragma unroll
-        for (int j = 0; j < kResidualSums; j++) out[j] = v[j];
+        for (int j = 0; j < kResidualSums; j++) {
+            out[j] = v[j];
+            if (host) host[j] = v[j];
+        }
+        if (host) host[kHostStatus] = (double)*err;
+    }
 }
 
 // Mass renormalisation.  With the Eq. 18 force and the pressure read as
@@ -2161,8 +2171,8 @@ __global__ void rescale_kernel(const StepArgs<S> a, S *f0, S *f1, const double *
 // Nusselt number (Eq. 90) along the west (hot) and east (cold) walls in FP64:
 // local values into loc[0..ny), trapezoid means into out[0], out[1].
 template <class S>
-__global__ void __launch_bounds__(256) nusselt_kernel(const StepArgs<S> a, double H, double dT,
-                                                      double *loc, double *out) {
+__global__ void __launch_bounds__(256) nusselt_kernel(const StepArgs<S> a, double H, double dT, double *loc,
+                                                      double *out, double *host) {
     __shared__ double red[2][8];
     double sh = 0.0, sc = 0.0;
     const int nx = a.nx;
@@ -2173,6 +2183,7 @@ __global__ void __launch_bounds__(256) nusselt_kernel(const StepArgs<S> a, doubl
         const double nh = -H * (-3.0 * t0 + 4.0 * t1 - t2) / (2.0 * dT);
         const double nc = -H * (3.0 * e0 - 4.0 * e1 + e2) / (2.0 * dT);
         loc[j] = nh;
+        if (host) host[kHostLocal + j] = nh;
         const double w = (j == 0 || j == a.ny - 1) ? 0.5 : 1.0;
         sh += w * nh;
         sc += w * nc;
@@ -2196,6 +2207,11 @@ __global__ void __launch_bounds__(256) nusselt_kernel(const StepArgs<S> a, doubl
         }
         out[0] = a0 / H;
         out[1] = a1 / H;
+        if (host) {
+            host[0] = a0 / H;
+            host[1] = a1 / H;
+            host[kHostStatus] = (double)*a.err;
+        }
     }
 }
 

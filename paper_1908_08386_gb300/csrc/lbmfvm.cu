@@ -304,6 +304,7 @@ struct lbmfvm {
     double nu, alpha, gbeta, tau, t_ref, force[2];
     unsigned char *base;
     bool owns;
+    double *host;     // page-locked, device-mapped results (kHost*), read after one synchronisation
     cudaStream_t user;
     cudaStream_t s;
     cudaEvent_t ev_in, ev_out;
@@ -662,15 +663,65 @@ void launch_residual(lbmfvm_t *h, int update_only) {
     double *sv = su + (size_t)h->grid.nx * h->grid.ny;
     double *red = reinterpret_cast<double *>(h->base + h->L.red);
     residual_kernel<S><<<kResidualBlocks, 256, 0, h->s>>>(a, direct, su, sv, red, update_only);
-    if (!update_only) residual_finish_kernel<<<1, 32, 0, h->s>>>(red, kResidualBlocks, red + kRedTot);
+    if (!update_only)
+        residual_finish_kernel<<<1, 32, 0, h->s>>>(red, kResidualBlocks, red + kRedTot, a.err, h->host);
 }
 
 template <class S, class O>
-void launch_fields(lbmfvm_t *h, int which, O *o0, O *o1) {
+void launch_fields(lbmfvm_t *h, O *const o[4]) {
     int direct;
     StepArgs<S> a = read_args<S>(h, direct);
     dim3 block(32, 8), grid((h->grid.nx + 31) / 32, (h->grid.ny + 7) / 8);
-    fields_kernel<S, O><<<grid, block, 0, h->s>>>(a, direct, which, o0, o1);
+    fields_kernel<S, O><<<grid, block, 0, h->s>>>(a, direct, o[0], o[1], o[2], o[3], h->host + kHostStatus);
+}
+
+// Whether a field kernel may write straight to the caller's arrays: memory of
+// this device, aligned for its element, no two the same.
+template <class O>
+bool writable_here(O *const o[4]) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    for (int i = 0; i < 4; i++) {
+        if (!o[i]) continue;
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, o[i]) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (at.type != cudaMemoryTypeDevice || at.device != dev || reinterpret_cast<uintptr_t>(o[i]) % sizeof(O))
+            return false;
+        for (int j = 0; j < i; j++)
+            if (o[j] == o[i]) return false;
+    }
+    return true;
+}
+
+// Fields by launch(outputs): straight into device arrays of the caller in one
+// pass, else through the staging area (two doubles a node).
+template <class O, class Launch>
+cudaError_t copy_fields(lbmfvm_t *h, size_t n, O *const outs[4], Launch launch) {
+    if (writable_here(outs)) {
+        launch(outs);
+        return cudaGetLastError();
+    }
+    O *st = reinterpret_cast<O *>(h->base + h->L.stage);
+    const int per = 2 * sizeof(double) / sizeof(O);  // fields the staging area holds
+    for (int f = 0; f < 4; f += per) {
+        O *part[4] = {nullptr, nullptr, nullptr, nullptr};
+        bool any = false;
+        for (int i = f; i < f + per; i++)
+            if (outs[i]) {
+                part[i] = st + (size_t)(i - f) * n;
+                any = true;
+            }
+        if (!any) continue;
+        launch(part);
+        cudaError_t e = cudaGetLastError();
+        for (int i = f; i < f + per && e == cudaSuccess; i++)
+            if (outs[i]) e = cudaMemcpyAsync(outs[i], part[i], n * sizeof(O), cudaMemcpyDefault, h->s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 template <class S>
@@ -678,7 +729,7 @@ void launch_nusselt(lbmfvm_t *h) {
     StepArgs<S> a = args_for<S>(h, h->parity);
     double *red = reinterpret_cast<double *>(h->base + h->L.red);
     const double dT = h->grid.t_wall[LBMFVM_SIDE_W] - h->grid.t_wall[LBMFVM_SIDE_E];
-    nusselt_kernel<S><<<1, 256, 0, h->s>>>(a, (double)(h->grid.ny - 1), dT, red + kRedLocal, red + kRedNu);
+    nusselt_kernel<S><<<1, 256, 0, h->s>>>(a, (double)(h->grid.ny - 1), dT, red + kRedLocal, red + kRedNu, h->host);
 }
 
 // Mass renormalisation of the current state (both population buffers) from
@@ -1080,17 +1131,28 @@ int setup_kernels(lbmfvm_t *h) {
     return LBMFVM_OK;
 }
 
+int status_failure(lbmfvm_t *h, int word) {
+    CU(h, cudaMemsetAsync(h->base + h->L.err, 0, sizeof(int), h->s));
+    return fail(h, LBMFVM_ERR_TIMEOUT, "a device-side wait for staged data ran out (status %d)", word);
+}
+
+// Waits for the handle's stream; the last kernel on it has written its results
+// and the status word into h->host (one synchronisation and no copies: the two
+// copies and second synchronisation of small calls took most of their time,
+// 46-60 us of 64^2 ones).
+int wait_results(lbmfvm_t *h) {
+    CU(h, cudaStreamSynchronize(h->s));
+    const int word = (int)static_cast<volatile double *>(h->host)[kHostStatus];
+    return word ? status_failure(h, word) : LBMFVM_OK;
+}
+
 // A bounded device-side wait that ran out leaves a non-zero status word.
 int check_device_status(lbmfvm_t *h) {
     int word = 0;
     int *dev = reinterpret_cast<int *>(h->base + h->L.err);
     CU(h, cudaMemcpyAsync(&word, dev, sizeof(int), cudaMemcpyDeviceToHost, h->s));
     CU(h, cudaStreamSynchronize(h->s));
-    if (word) {
-        CU(h, cudaMemsetAsync(dev, 0, sizeof(int), h->s));
-        return fail(h, LBMFVM_ERR_TIMEOUT, "a device-side wait for staged data ran out (status %d)", word);
-    }
-    return LBMFVM_OK;
+    return word ? status_failure(h, word) : LBMFVM_OK;
 }
 
 // Autotuner of the TMA tile shape.  Each shape steps the handle's own grid
@@ -1385,6 +1447,13 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
         }
         h->owns = true;
     }
+    // (a batch's packed grid has one row of local Nusselt numbers per node row of its tallest cavity at most)
+    e = cudaHostAlloc(&h->host, (kHostLocal + (size_t)grid->ny) * sizeof(double), cudaHostAllocMapped);
+    if (e != cudaSuccess) {
+        h->host = nullptr;
+        fail(h, LBMFVM_ERR_NOMEM, "cudaHostAlloc failed: %s", cudaGetErrorString(e));
+        return bail(LBMFVM_ERR_NOMEM);
+    }
     std::vector<uint8_t> code = atlas ? atlas->codes : classify(*grid, mask, L.pitch);
     if (atlas) {
         h->atlas_cavs = atlas->cavs;
@@ -1419,19 +1488,15 @@ template <class O>
 int fields_impl(lbmfvm_t *h, O *rho, O *u, O *v, O *T) {
     if (!h) return fail_thread(LBMFVM_ERR_ARG, "handle is NULL");
     const size_t n = (size_t)h->grid.nx * h->grid.ny;
-    O *st = reinterpret_cast<O *>(h->base + h->L.stage);
     if (int r = join_in(h)) return r;
-    O *outs[2][2] = {{rho, u}, {v, T}};
-    for (int which = 0; which < 2; which++) {
-        if (!outs[which][0] && !outs[which][1]) continue;
-        DISPATCH(h, launch_fields, h, which, st, st + n);
-        CU(h, cudaGetLastError());
-        for (int i = 0; i < 2; i++)
-            if (outs[which][i])
-                CU(h, cudaMemcpyAsync(outs[which][i], st + i * n, n * sizeof(O), cudaMemcpyDefault, h->s));
+    O *const outs[4] = {rho, u, v, T};
+    if (!rho && !u && !v && !T) {
+        CU(h, cudaStreamSynchronize(h->s));
+        if (int r = check_device_status(h)) return r;
+        return join_out(h);
     }
-    CU(h, cudaStreamSynchronize(h->s));
-    if (int r = check_device_status(h)) return r;
+    CU(h, copy_fields<O>(h, n, outs, [&](O *const *o) { DISPATCH(h, launch_fields, h, o); }));
+    if (int r = wait_results(h)) return r;
     return join_out(h);
 }
 
@@ -1657,16 +1722,22 @@ int lbmfvm_nusselt(lbmfvm_t *h, double *mean_hot, double *local_hot, double *mea
     if (int r = join_in(h)) return r;
     DISPATCH(h, launch_nusselt, h);
     CU(h, cudaGetLastError());
-    double *red = reinterpret_cast<double *>(h->base + h->L.red);
-    double means[2];
-    CU(h, cudaMemcpyAsync(means, red + kRedNu, sizeof(means), cudaMemcpyDeviceToHost, h->s));
-    if (local_hot)
-        CU(h, cudaMemcpyAsync(local_hot, red + kRedLocal, h->grid.ny * sizeof(double),
-                              cudaMemcpyDefault, h->s));
-    CU(h, cudaStreamSynchronize(h->s));
+    const size_t row = h->grid.ny * sizeof(double);
+    bool local_device = false;
+    if (local_hot) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, local_hot) != cudaSuccess) cudaGetLastError();
+        else local_device = at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+        if (local_device)
+            CU(h, cudaMemcpyAsync(local_hot, reinterpret_cast<double *>(h->base + h->L.red) + kRedLocal, row,
+                                  cudaMemcpyDefault, h->s));
+    }
+    const int status = wait_results(h);
+    const double means[2] = {h->host[0], h->host[1]};
+    if (local_hot && !local_device) std::memcpy(local_hot, h->host + kHostLocal, row);
     if (mean_hot) *mean_hot = means[0];
     if (mean_cold) *mean_cold = means[1];
-    if (int r = check_device_status(h)) return r;
+    if (status) return status;
     if (!std::isfinite(means[0]) || !std::isfinite(means[1]))
         return fail(h, LBMFVM_ERR_DIVERGED, "non-finite Nusselt number");
     return join_out(h);
@@ -1677,14 +1748,11 @@ int lbmfvm_residual(lbmfvm_t *h, double *r) {
     if (int e = join_in(h)) return e;
     DISPATCH(h, launch_residual, h, 0);
     CU(h, cudaGetLastError());
-    double sums[2];
-    double *red = reinterpret_cast<double *>(h->base + h->L.red);
-    CU(h, cudaMemcpyAsync(sums, red + kRedTot, sizeof(sums), cudaMemcpyDeviceToHost, h->s));
-    CU(h, cudaStreamSynchronize(h->s));
-    if (int e = check_device_status(h)) {
+    if (int e = wait_results(h)) {
         *r = NAN;
         return e;
     }
+    const double sums[2] = {h->host[0], h->host[1]};
     if (!std::isfinite(sums[0]) || !std::isfinite(sums[1])) {
         *r = NAN;
         return fail(h, LBMFVM_ERR_DIVERGED, "non-finite velocity in the residual");
@@ -1766,6 +1834,7 @@ void lbmfvm_destroy(lbmfvm_t *h) {
     if (h->s) cudaStreamSynchronize(h->s);
     if (h->graph) cudaGraphExecDestroy(h->graph);
     if (h->owns && h->base) cudaFree(h->base);
+    if (h->host) cudaFreeHost(h->host);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->ev_out) cudaEventDestroy(h->ev_out);
     if (h->s) cudaStreamDestroy(h->s);
