@@ -168,8 +168,9 @@ typedef struct {
                                per SM); 128x8, 1024, 2/3, 3; 32x16, 256 + 64 ring
                                threads (two warps that take the one-node ring's
                                moments and issue the copies; two blocks per SM),
-                               3/3, 2; 64x16, 512 + 96 ring threads, 3/3, 2.  Of
-                               these, 1, 4 and 5 take pairs of nodes per thread.
+                               3/3, 2; 64x16, 512 + 96 ring threads and a warp that
+                               issues the copies, 3/3, 2.  Of these, 1, 4 and 5
+                               take pairs of nodes per thread.
                                64-bit storage: 64x8, 256, 2;
                                32x8, 256, 3; 32x16, 512, 2; 32x8, 256, 2 (two
                                blocks per SM); 32x8, 256 + 64 ring threads, 3;
@@ -177,7 +178,9 @@ typedef struct {
                                LBMFVM_TMA_DEFAULT: for a grid with fewer tiles
                                than the GPU has SMs, 2 (32- and 16-bit storage)
                                or 4 (64-bit), which spread it over more SMs;
-                               otherwise 4 (32- and 16-bit) or 3 (64-bit): the
+                               otherwise 4 for 32-bit storage whose population
+                               buffers and temperature planes fit in the L2, 5
+                               beyond it and for 16-bit storage, 3 for 64-bit: the
                                fastest measured on 64^2 to 4096^2 cavities.
                                LBMFVM_TMA_AUTOTUNE times every shape (a
                                captured graph of 32 launches, replayed twice)

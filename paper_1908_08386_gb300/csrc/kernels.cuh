@@ -840,6 +840,10 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -914,13 +918,20 @@ __device__ __forceinline__ void load_2d(void *dst, const CUtensorMap *map, uint6
 // the THREADS compute threads all carry the same load into each tile's block
 // barrier; with 0 the first compute threads also take the ring and thread 0
 // issues.
+//
+// PW adds a warp that only issues the copies: a tile's store goes out as soon
+// as its compute warps have written it and the refill follows it, without
+// holding up the ring warps before the next tile's barrier.  Where two blocks
+// share an SM its registers cost more than that gives.
 template <class S, int TW_, int TH_, int STAGES_, int THREADS_, int MINB_ = 1, int THALO_ = 1, int RT_ = 0,
-          int FHALO_ = 2>
+          int FHALO_ = 2, bool PW_ = false>
 struct TmaTile {
     using TC = typename Compute<S>::type;  // temperature and ring element
     static constexpr int TW = TW_, TH = TH_, STAGES = STAGES_, THREADS = THREADS_;
     static constexpr int RING_THREADS = RT_;
-    static constexpr int BLOCK = THREADS_ + RT_;       // threads per block
+    static constexpr int CONSUMERS = THREADS_ + RT_;
+    static constexpr bool PW = PW_;                     // a warp of its own issues the copies
+    static constexpr int BLOCK = CONSUMERS + (PW ? 32 : 0);  // threads per block
     static constexpr int MINB = MINB_;             // blocks per SM the register budget must allow
     static constexpr int THALO = THALO_;
     static constexpr int NPT = TW * TH / THREADS;  // own nodes per thread
@@ -955,7 +966,7 @@ struct TmaTile {
     static constexpr uint32_t RING_OFF = STAGES * STAGE_BYTES;
     static constexpr uint32_t RING_BYTES = align128(2u * RH * RW * (uint32_t)sizeof(TC));  // u, v of tile + ring
     static constexpr uint32_t BAR_OFF = RING_OFF + 2u * RING_BYTES;      // two ring buffers
-    static constexpr uint32_t HDR_OFF = BAR_OFF + align128(8u * STAGES + 16u);
+    static constexpr uint32_t HDR_OFF = BAR_OFF + align128(20u * STAGES + 16u);  // full, done, flags, valid
     static constexpr uint32_t SMEM_BYTES = HDR_OFF + STAGES * (uint32_t)sizeof(TileHeader);
     static_assert(SMEM_BYTES <= 232448u, "tile configuration exceeds 227 KB of shared memory");
     static_assert(OT_OFF + OT_BYTES <= F_BYTES, "results must fit in the staged population bytes");
@@ -971,7 +982,7 @@ struct TmaTile {
     static_assert(FHALO == 2 || FHALO == 3, "population halo of two or three rows");
     // the same tile with a temperature box of h halo rows
     template <int h>
-    using WithTHalo = TmaTile<S, TW_, TH_, STAGES_, THREADS_, MINB_, h, RT_, FHALO_>;
+    using WithTHalo = TmaTile<S, TW_, TH_, STAGES_, THREADS_, MINB_, h, RT_, FHALO_, PW_>;
 };
 
 // Energy update of a launch of the TMA kernel: the central face values of
@@ -991,12 +1002,14 @@ template <class S> struct TmaConfig<S, 2> { using G = TmaTile<S, 64, 8, sizeof(S
 template <class S> struct TmaConfig<S, 3> { using G = TmaTile<S, 128, 8, sizeof(S) == 4 ? 2 : 3, 1024, 1, 1, 0, 3>; };
 // 32 x 16 with two ring warps (which also issue the copies), two blocks per
 // SM, so that one block's barrier, loads and stores overlap the other's
-// arithmetic; 64 x 16 with three ring warps, one block per SM.  Us per step,
+// arithmetic; 64 x 16 with three ring warps and a copying warp, one block per
+// SM.  Us per step,
 // single nodes in 64 x 16 / pairs in 64 x 16 / pairs in 32 x 16: 1024^2 FP32
 // 18.1 / 17.0 / 15.4-16.3, FP16 17.0 / 15.1 / 14.6-15.3; 4096^2 FP32 236 / 222 /
-// 213, FP16 212 / 175 / 171-178
+// 213, FP16 212 / 175 / 171-178; with the copying warp (shape 5): 1024^2 FP32
+// 16.6, FP16 14.6, 4096^2 210 and 167.5 (32 x 16 with one: 17.0, 15.6, 227, 189)
 template <class S> struct TmaConfig<S, 4> { using G = TmaTile<S, 32, 16, 3, 256, 2, 1, 64, 2>; };
-template <class S> struct TmaConfig<S, 5> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 96, 2>; };
+template <class S> struct TmaConfig<S, 5> { using G = TmaTile<S, 64, 16, 3, 512, 1, 1, 96, 2, true>; };
 // 64-bit storage: a 32 x 8 tile stages 43 KB, a 64 x 8 tile 78 KB.
 template <> struct TmaConfig<double, 0> { using G = TmaTile<double, 64, 8, 2, 256>; };
 template <> struct TmaConfig<double, 1> { using G = TmaTile<double, 32, 8, 3, 256>; };
@@ -1079,6 +1092,8 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::BAR_OFF);
     int *abort_flag = reinterpret_cast<int *>(smem + G::BAR_OFF + 8 * G::STAGES);
     volatile int *known = abort_flag + 1;  // tiles this block is known to have
+    uint64_t *done = reinterpret_cast<uint64_t *>(smem + G::BAR_OFF + 8 * G::STAGES + 16);  // results written
+    volatile int *valid = reinterpret_cast<int *>(done + G::STAGES);  // stage holds a tile (0: the sequence has ended)
     TileHeader *hdrs = reinterpret_cast<TileHeader *>(smem + G::HDR_OFF);
 
     const int tid = threadIdx.x;
@@ -1123,7 +1138,10 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
     };
 
     if (tid == 0) {
-        for (int s = 0; s < G::STAGES; s++) tma::mbar_init(&bars[s], 1);
+        for (int s = 0; s < G::STAGES; s++) {
+            tma::mbar_init(&bars[s], 1);
+            if (G::PW) tma::mbar_init(&done[s], G::THREADS / 32);
+        }
         *abort_flag = 0;
         *known = 0;
         tma::fence_mbar_init();
@@ -1136,11 +1154,84 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
     // Without a programmatic predecessor the wait returns at once.
     if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (G::PW) {
+        if (tid >= G::CONSUMERS) {
+            // The copying thread of its own warp, off the other warps' path:
+            // stages filled in turn, each result stored as soon as the compute
+            // warps have written it, its stage refilled once the store has
+            // read it; a stage marked invalid ends the block's sequence.
+            if (tid > G::CONSUMERS) return;
+            if (blockIdx.x == 0) *ctr_next = 0;
+            int issued = 0, ticket = -1;
+            bool ended = false;
+            auto finish = [&](int k) {
+                valid[k % G::STAGES] = 0;
+                tma::mbar_arrive(&bars[k % G::STAGES]);
+                ended = true;
+            };
+            for (int k = 0; k < G::STAGES && !ended; k++) {
+                const int t = fixed_tile(k);
+                if (t < 0) {
+                    finish(k);
+                } else {
+                    valid[k] = 1;
+                    if (!(a.stall && blockIdx.x == 0 && k == 0)) issue(k, t, origin(t));
+                    issued++;
+                }
+            }
+            if (!ended && G::STAGES >= nfix) ticket = atomicAdd(ctr, 1);
+            for (int k = 0; k < issued; k++) {
+                // the tile after next for this stage, its origin and the next
+                // ticket, while the compute warps work
+                const int m = k + G::STAGES;
+                int t = -1;
+                int2 o = make_int2(0, 0);
+                if (!ended) {
+                    if (m < nfix) {
+                        t = fixed_tile(m);
+                    } else {
+                        t = nfix * (int)gridDim.x + ticket;
+                        if (t >= ntiles) t = -1;
+                    }
+                    if (t >= 0) {
+                        o = origin(t);
+                        if (m + 1 >= nfix) ticket = atomicAdd(ctr, 1);
+                    }
+                }
+                bool ok = false;
+                const uint64_t t0 = tma::globaltimer();
+                for (uint32_t it = 0; !*(volatile int *)abort_flag; it++) {
+                    if ((ok = tma::mbar_try_wait(&done[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u))) break;
+                    if ((it & 63u) == 63u && tma::globaltimer() - t0 > 2 * kWaitLimitNs) break;
+                }
+                if (!ok) {
+                    // let the copies already in flight land before the block exits
+                    for (int j = k; j < issued; j++)
+                        if (!(a.stall && blockIdx.x == 0 && j == 0))
+                            tma::mbar_wait_bounded(&bars[j % G::STAGES], (uint32_t)(j / G::STAGES) & 1u, kWaitLimitNs / 2);
+                    atomicOr(a.err, kErrTimeout);
+                    break;
+                }
+                store_tile(k);
+                if (ended) continue;
+                tma::bulk_wait_read();
+                if (t < 0) {
+                    finish(m);
+                } else {
+                    valid[m % G::STAGES] = 1;
+                    issue(m, t, o);
+                    issued++;
+                }
+            }
+            tma::bulk_wait_all();
+            return;
+        }
+    }
     // the issuing thread: the next tile to load (index, origin), the ticket
     // in flight, loads issued
     int pre_t = -1, ticket = -1, issued = 0;
     int2 pre_o = make_int2(0, 0);
-    if (tid == PROD) {
+    if (!G::PW && tid == PROD) {
         if (blockIdx.x == 0) *ctr_next = 0;
         int k = 0;
         for (; k < G::STAGES && fixed_tile(k) >= 0; k++) {
@@ -1157,15 +1248,17 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
         }
         *known = k;
     }
-    __syncthreads();
+    if constexpr (!G::PW) __syncthreads();
 
-    for (int k = 0; k < *known; k++) {
+    for (int k = 0; G::PW || k < *known; k++) {
         unsigned char *stg = stage(k);
         const bool landed = tma::mbar_wait_bounded(&bars[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u, kWaitLimitNs);
         if (!landed) {
             atomicOr(abort_flag, 1);
             atomicOr(a.err, kErrTimeout);
         }
+        if constexpr (G::PW)
+            if (landed && !valid[k % G::STAGES]) break;  // for every thread alike
         // a stage that never landed has no header: use a harmless one (the
         // block leaves at the next barrier)
         const TileHeader hd = landed ? hdrs[k % G::STAGES] : TileHeader{};
@@ -1397,9 +1490,10 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                 }
             }
         }
-        __syncthreads();
-        if (*abort_flag) {
-            if (tid == PROD) {
+        if constexpr (G::PW) asm volatile("bar.sync 1, %0;" ::"n"(G::CONSUMERS) : "memory");
+        else __syncthreads();
+        if (*(volatile int *)abort_flag) {
+            if (!G::PW && tid == PROD) {
                 // let the copies already in flight land before the block exits
                 for (int j = k + 1; j < issued; j++)
                     tma::mbar_wait_bounded(&bars[j % G::STAGES], (uint32_t)(j / G::STAGES) & 1u, kWaitLimitNs / 2);
@@ -1407,7 +1501,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
             }
             return;
         }
-        if (tid == PROD && k > 0) store_tile(k - 1);
+        if (!G::PW && tid == PROD && k > 0) store_tile(k - 1);
 
         // Phase B: energy balance and collision of the own nodes; results go
         // to the stage's (now dead) population bytes.  Inert nodes keep T.
@@ -1511,7 +1605,13 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                 collide<C>(g[j], dr[j], uu[j], vv[j], omega, fx, Gy, [&](int q, C v) { st(of + q * OPLANE, v); });
             }
         }
-        if (tid == PROD && k > 0 && pre_t >= 0) {
+        if constexpr (G::PW) {
+            if (computes) {
+                __syncwarp();
+                if ((tid & 31) == 0) tma::mbar_arrive(&done[k % G::STAGES]);
+            }
+        }
+        if (!G::PW && tid == PROD && k > 0 && pre_t >= 0) {
             tma::bulk_wait_read();  // the results of tile k-1 have left its stage
             issue(k - 1 + G::STAGES, pre_t, pre_o);
             issued = k + G::STAGES;
@@ -1531,6 +1631,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
             }
         }
     }
+    if constexpr (G::PW) return;
     const int count = *known;
     __syncthreads();
     if (tid == PROD && count > 0) {

@@ -1377,23 +1377,29 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
     h->tile_y = opts.tile_y ? opts.tile_y : 8;
     h->use_tma = tma_ok && opts.kernel != LBMFVM_KERNEL_GENERIC;
     // the default shapes are the fastest measured ones: two blocks of 32 x 16
-    // per SM with ring warps for 32- and 16-bit storage, two blocks of 32 x 8
-    // per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
+    // per SM with ring warps for 32-bit storage that fits the L2 (1024^2: 16.0 us
+    // against 16.6), 64 x 16 with a copying warp beyond it (4096^2: 210 against
+    // 213) and for 16-bit storage (1024^2: 14.6 against 15.3; 4096^2: 167.5
+    // against 177.5), two blocks of 32 x 8 per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
     // SMs is bound by the latency of one tile, not by the SMs' throughput, and
     // takes the smaller tiles that spread it over more SMs: 64 x 8 (two blocks
     // per SM) for 32- and 16-bit storage, 32 x 8 with ring warps for 64-bit.
     int shape_default = 3;
     {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
+        int dev = 0, l2 = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 0;
+            l2 = sms = 0;
         const long long tiles = store_size(opts.store) == 8
                                     ? (long long)((grid->nx + 31) / 32) * ((grid->ny + 7) / 8)
                                     : (long long)((grid->nx + 63) / 64) * ((grid->ny + 15) / 16);
         const bool small = tiles < sms;
-        if (store_size(opts.store) == 8) shape_default = small ? 4 : 3;
-        else shape_default = small ? 2 : 4;
+        if (store_size(opts.store) == 8) {
+            shape_default = small ? 4 : 3;
+        } else {
+            const size_t state = 2 * (9 * store_size(opts.store) + temp_size(opts.store)) * (size_t)L.plane;
+            shape_default = small ? 2 : store_size(opts.store) == 4 && state <= (size_t)l2 ? 4 : 5;
+        }
     }
     const bool own_shape = opts.tma_config == LBMFVM_TMA_AUTOTUNE || opts.tma_config == LBMFVM_TMA_DEFAULT;
     h->tma_config = own_shape ? shape_default : opts.tma_config;
