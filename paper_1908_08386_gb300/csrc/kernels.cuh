@@ -394,7 +394,7 @@ __device__ __forceinline__ void nee(C g[9], C &drho, C &ux, C &uy, C uw, C vw) {
     pair(2, 4, vw, uy);
     pair(5, 7, uw + vw, ux + uy);
     pair(6, 8, vw - uw, uy - ux);
-    if constexpr (std::is_same<C, dsf>::value) {
+    if constexpr (std::is_same<C, dsf>::value || std::is_same<C, double>::value) {
         // the non-equilibrium part carries no mass and no momentum, so the
         // node's density is the partner's and its velocity the wall's
         ux = uw;

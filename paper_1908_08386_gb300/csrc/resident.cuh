@@ -9,8 +9,8 @@
 // step, one launch per step -> resident): FP32 64^2 3.68 -> 1.68, 128^2 3.98 ->
 // 1.89, 256^2 4.62 -> 2.16, 384^2 4.93 -> 3.19, 512^2 7.55 -> 5.89; FP16 256^2
 // 4.45 -> 2.28; double-single 64^2 5.82 -> 3.39, 128^2 5.76 -> 3.04, 192^2 5.95 ->
-// 3.57, 256^2 8.5 -> 6.3; FP64 64^2 21.0 -> 9.3, 128^2 21.0 -> 11.7, 192^2 21.1 ->
-// 19.3; 512 x 384 with QUICK and two sub-steps (four launches) 27.2 -> 10.3.
+// 3.57, 256^2 8.5 -> 6.3; FP64 64^2 21.0 -> 5.0, 128^2 21.0 -> 9.1, 192^2 21.1 ->
+// 15.6; 512 x 384 with QUICK and two sub-steps (four launches) 27.2 -> 10.3.
 // What bounds it now: the exchange (about 1.1 us) and, for the 64-bit types,
 // the dependent chain of one node's operations.
 //
@@ -48,7 +48,10 @@ struct ResTile {
     using C = typename Compute<S>::type;
     static constexpr int TW = TW_, TH = TH_, NT = NT_, RT = RT_;
     static constexpr int BLOCK = NT + RT;        // tile threads, then ring threads
-    static constexpr int NPT = TW * TH / NT;     // own nodes per tile thread
+    // Four threads per node (small FP64 tiles, see quad_moments): one direction
+    // pair and one face each.
+    static constexpr bool QUAD = NT == 4 * TW * TH;
+    static constexpr int NPT = QUAD ? 1 : TW * TH / NT;  // own nodes per tile thread
     static constexpr int FW = TW + 4, FH = TH + 4, PL = FW * FH;  // staged box: two nodes around the tile
     static constexpr int RW = TW + 2, RH = TH + 2;
     static constexpr int NRING = 2 * TW + 2 * TH;                 // ring nodes a face can touch (no corners)
@@ -71,7 +74,7 @@ struct ResTile {
     static constexpr size_t U_OFF = T_OFF + a16(2 * (size_t)PL * sizeof(C));
     static constexpr size_t W_OFF = U_OFF + a16(2 * (size_t)RW * RH * sizeof(C));
     static constexpr size_t SMEM = W_OFF + a16(10 * sizeof(C));
-    static_assert(TW * TH % NT == 0 && NT % TW == 0 && NT % 32 == 0 && RT % 32 == 0 && BLOCK <= 1024, "threads");
+    static_assert((QUAD || (TW * TH % NT == 0 && NT % TW == 0)) && NT % 32 == 0 && RT % 32 == 0 && BLOCK <= 1024, "threads");
     static_assert(SMEM <= 230000, "shared memory");
 };
 
@@ -197,6 +200,66 @@ struct Packet {
 
 }  // namespace mail
 
+// A node's arithmetic split over four neighbouring lanes, s = 0..3.  An FP64
+// instruction holds its quarter of an SM for some 80 cycles whatever it
+// computes, and a 32-node tile is one warp: one quarter works, the others wait.
+// With a lane per direction pair and per face a warp executes about 70 of them
+// a step instead of 170, on all four quarters.  Same operations in the same
+// order, so the same bits.  64^2 FP64: 8.6 -> 5.0 us per step.  Larger tiles
+// fill the quarters as they are.
+template <class C>
+__device__ __forceinline__ C quad_pick(int s, C a, C b, C c, C d) {
+    return s < 2 ? (s == 0 ? a : b) : (s == 2 ? c : d);
+}
+template <class C>
+__device__ __forceinline__ C quad_get(C v, int s) {
+    return __shfl_sync(0xffffffffu, v, s, 4);
+}
+template <class C>
+__device__ __forceinline__ void quad_moments(const C g[9], int s, C &drho, C &ux, C &uy) {
+    const C p = quad_pick(s, g[0], g[2], g[4], g[6]) + quad_pick(s, g[1], g[3], g[5], g[7]);
+    const C q = (quad_pick(s, g[1], g[3], g[2], g[4]) + quad_pick(s, g[5], g[6], g[5], g[7])) +
+                quad_pick(s, g[8], g[7], g[6], g[8]);
+    drho = ((quad_get(p, 0) + quad_get(p, 1)) + (quad_get(p, 2) + quad_get(p, 3))) + g[8];
+    const C jx = quad_get(q, 0) - quad_get(q, 1), jy = quad_get(q, 2) - quad_get(q, 3);
+    const C inv = recip(C(1) + drho);
+    ux = mul_r(jx, inv);
+    uy = mul_r(jy, inv);
+}
+// nee for the lane's pair (f, b) and the rest population.
+template <class C>
+__device__ __forceinline__ void quad_nee(C &g0, C &f, C &b, int s, C drho, C &ux, C &uy, C uw, C vw) {
+    const C rho = C(1) + drho;
+    const C dP0 = mul_r(C(-1.5f), fma_c(uw, uw, mul_r(vw, vw)) - fma_c(ux, ux, mul_r(uy, uy)));
+    if (s == 0) g0 = fma_c(mul_r(rho, wq<C>(0)), dP0, g0);
+    const C euw = quad_pick(s, uw, vw, uw + vw, vw - uw), euf = quad_pick(s, ux, uy, ux + uy, uy - ux);
+    const C A = fma_c(C(4.5f), fma_c(euw, euw, -mul_r(euf, euf)), dP0), B = triple(euw - euf);
+    const C rw = mul_r(rho, s < 2 ? wq<C>(1) : wq<C>(5));
+    f = fma_c(rw, A + B, f);
+    b = fma_c(rw, A - B, b);
+    ux = uw;
+    uy = vw;
+}
+// collide for the lane's pair, store(q, value); the rest population by lane 0.
+template <class C, class Store>
+__device__ __forceinline__ void quad_collide(C g0, C f, C b, int s, C drho, C ux, C uy, C omega, C Gx, C Gy,
+                                             Store store) {
+    const C rho = C(1) + drho;
+    const C P0 = mul_r(C(-1.5f), fma_c(ux, ux, mul_r(uy, uy)));
+    const C c = mul_r(C(3), rho);
+    const C sx = mul_r(c, Gx), sy = mul_r(c, Gy);
+    const C nGu = -fma_c(sx, ux, mul_r(sy, uy));
+    const C om1 = C(1) - omega;
+    auto out = [&](int q, C w, C gq, C P, C z) {
+        store(q, fma_c(om1, gq, mul_r(w, fma_c(P, fma_c(omega, rho, z), fma_c(omega, drho, z)))));
+    };
+    const C eu = quad_pick(s, ux, uy, ux + uy, uy - ux), es = quad_pick(s, sx, sy, sx + sy, sy - sx);
+    const C A = fma_c(C(4.5f), mul_r(eu, eu), P0), B = triple(eu), w = s < 2 ? wq<C>(1) : wq<C>(5);
+    out(s < 2 ? 1 + s : 3 + s, w, f, A + B, nGu + es);
+    out(s < 2 ? 3 + s : 5 + s, w, b, A - B, nGu - es);
+    if (s == 0) out(0, wq<C>(0), g0, P0, nGu);
+}
+
 // Arguments of a resident launch: steps from the state a.fin, a.Tin to a.fout,
 // a.Tout (other buffers), on one tile per block.
 template <class S>
@@ -282,6 +345,10 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             for (int l = 0; l < 2; l++) r.ctr[l][0] = r.ctr[l][1] = 0;
     }
 
+    // own node j of this thread, and its lane of the four that share it
+    auto own_node = [&](int j) { return G::QUAD ? tid >> 2 : tid + j * G::NT; };
+    const int lane4 = tid & 3;
+
     // Own nodes: code, face flags, far-face flags (QUICK), wall side.
     const bool computes = tid < G::NT;
     uint32_t info[NPT];
@@ -289,7 +356,7 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
 #pragma unroll
     for (int j = 0; j < NPT; j++) {
         info[j] = kDead;
-        const int i = tid + j * G::NT, ly = i / TW, lx = i - ly * TW;
+        const int i = own_node(j), ly = i / TW, lx = i - ly * TW;
         if (computes && in_cavity(lx, ly)) {
             const long long k = org + (long long)ly * pitch + lx;
             const uint8_t c = decode(r.a.code[k]);
@@ -450,13 +517,25 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
     for (int k = 0; k < r.nsteps; k++) {
         // Phase A: moments of the own nodes (kept in registers) and of the ring.
         C g[NPT][9], dr[NPT], uu[NPT], vv[NPT], Tn[NPT];
+        C qf, qb;  // the lane's pair of populations (four threads per node)
         if (computes) {
 #pragma unroll
             for (int j = 0; j < NPT; j++) {
-                const int i = tid + j * G::NT, ly = i / TW, lx = i - ly * TW;
+                const int i = own_node(j), ly = i / TW, lx = i - ly * TW;
                 const uint32_t c = info[j];
                 const int kind = c & 3;
-                if (kind != KIND_SOLID) {
+                if constexpr (G::QUAD) {
+                    const int d = kind == KIND_WALL ? partner_dir((uint8_t)c) : 0;
+                    pull(lx + cx_rt(d), ly + cy_rt(d), g[j]);  // inert nodes hold zeros
+                    quad_moments<C>(g[j], lane4, dr[j], uu[j], vv[j]);
+                    qf = quad_pick(lane4, g[j][1], g[j][2], g[j][5], g[j][6]);
+                    qb = quad_pick(lane4, g[j][3], g[j][4], g[j][7], g[j][8]);
+                    if (kind == KIND_WALL) {
+                        const int sd = (c >> 20) & 7;
+                        quad_nee<C>(g[j][0], qf, qb, lane4, dr[j], uu[j], vv[j], wall[2 * sd], wall[2 * sd + 1]);
+                    }
+                    if (kind == KIND_SOLID) uu[j] = vv[j] = C(0);
+                } else if (kind != KIND_SOLID) {
                     // a warp of fluid and wall nodes pulls and sums once (a
                     // wall node from its partner)
                     const int d = kind == KIND_WALL ? partner_dir((uint8_t)c) : 0;
@@ -502,12 +581,32 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
 #pragma unroll
                 for (int j = 0; j < NPT; j++) {
                     const uint32_t c = info[j];
-                    if ((c & 3) == KIND_SOLID) continue;
-                    const int i = tid + j * G::NT, ly = i / TW, lx = i - ly * TW;
+                    if (!(G::QUAD && !GENERAL) && (c & 3) == KIND_SOLID) continue;
+                    const int i = own_node(j), ly = i / TW, lx = i - ly * TW;
                     const int t = fi(lx, ly), rr = (ly + 1) * RW + lx + 1, th = (c >> 6) & 3;
                     const C TP = Tc[t];
                     C t1 = TP;
-                    if (th == TH_FV) {
+                    if constexpr (G::QUAD && !GENERAL) {
+                        // lanes E, W, N, S: one face each, summed as fv_update does
+                        const bool vert = lane4 >= 2, minus = (lane4 & 1) == 0;
+                        const int step = lane4 & 1 ? -1 : 1;
+                        const C Tb = Tc[t + step * (vert ? FW : 1)];
+                        const C wb = vert ? RV[rr + step * RW] : RU[rr + step], wP = vert ? vv[j] : uu[j];
+                        const C pr = mul_r(C(0.25f) * (wP + wb), TP + Tb);
+                        const uint32_t ff = c >> 8;
+                        const uint32_t bit = vert ? (minus ? FF_OPEN_N : FF_OPEN_S) : (minus ? FF_OPEN_E : FF_OPEN_W);
+                        const C f = ff & bit ? fma_c(alpha, Tb - TP, minus ? -pr : pr) : C(0);
+                        const C fe = quad_get(f, 0), fw = quad_get(f, 1), fn = quad_get(f, 2), fs = quad_get(f, 3);
+                        if (th == TH_FV) {
+                            const C ex = ((ff & FF_IN_W) ? C(0.5) : C(0)) + ((ff & FF_IN_E) ? C(0.5) : C(0));
+                            const C ey = ((ff & FF_IN_S) ? C(0.5) : C(0)) + ((ff & FF_IN_N) ? C(0.5) : C(0));
+                            const C inv_v = (ex < C(1) ? C(2) : C(1)) * (ey < C(1) ? C(2) : C(1));
+                            t1 = TP + (ey * (fe + fw) + ex * (fn + fs)) * inv_v;
+                        } else if (th == TH_OBSTACLE) {
+                            const int d = partner_dir((uint8_t)c);
+                            t1 = Tc[t + cy_rt(d) * FW + cx_rt(d)];
+                        }
+                    } else if (th == TH_FV) {
                         const uint32_t ff = c >> 8, far = c >> 16;
                         const C ex = ((ff & FF_IN_W) ? C(0.5) : C(0)) + ((ff & FF_IN_E) ? C(0.5) : C(0));
                         const C ey = ((ff & FF_IN_S) ? C(0.5) : C(0)) + ((ff & FF_IN_N) ? C(0.5) : C(0));
@@ -556,9 +655,16 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             for (int j = 0; j < NPT; j++) {
                 const uint32_t c = info[j];
                 if ((c & 3) == KIND_SOLID) continue;
-                const int i = tid + j * G::NT, ly = i / TW, lx = i - ly * TW;
+                const int i = own_node(j), ly = i / TW, lx = i - ly * TW;
                 const C Gy = fma_c(gbeta, Tn[j] - t_ref, fy);
-                if (last) {
+                if constexpr (G::QUAD) {
+                    const long long kk = org + (long long)ly * pitch + lx;
+                    S *out = last ? r.a.fout + kk : F + fi(lx, ly);
+                    const long long pl = last ? plane : PL;
+                    if (last) r.a.Tout[kk] = Tn[j];
+                    quad_collide<C>(g[j][0], qf, qb, lane4, dr[j], uu[j], vv[j], omega, fx, Gy,
+                                    [&](int q, C v) { st(out + q * pl, v); });
+                } else if (last) {
                     const long long kk = org + (long long)ly * pitch + lx;
                     S *out = r.a.fout + kk;
                     r.a.Tout[kk] = Tn[j];
@@ -608,14 +714,14 @@ template <class S> struct ResConfig<S, 2> { using G = ResTile<S, 32, 16, 512, 96
 template <class S> struct ResConfig<S, 3> { using G = ResTile<S, 32, 32, 512, 128>; };
 template <class S> struct ResConfig<S, 4> { using G = ResTile<S, 64, 32, 512, 128>; };
 template <class S> struct ResConfig<S, 5> { using G = ResTile<S, 64, 40, 512, 128>; };
-#define LBMFVM_RES_WIDE(S)                                                        \
-    template <> struct ResConfig<S, 0> { using G = ResTile<S, 8, 4, 32, 32>; };    \
+#define LBMFVM_RES_WIDE(S, QUAD)                                                     \
+    template <> struct ResConfig<S, 0> { using G = ResTile<S, 8, 4, 32 * QUAD, 32>; }; \
     template <> struct ResConfig<S, 1> { using G = ResTile<S, 8, 8, 64, 32>; };    \
     template <> struct ResConfig<S, 2> { using G = ResTile<S, 16, 8, 128, 64>; };  \
     template <> struct ResConfig<S, 3> { using G = ResTile<S, 32, 8, 256, 96>; };  \
     template <> struct ResConfig<S, 4> { using G = ResTile<S, 32, 16, 256, 96>; };
-LBMFVM_RES_WIDE(double)
-LBMFVM_RES_WIDE(dsf)
+LBMFVM_RES_WIDE(double, 4)
+LBMFVM_RES_WIDE(dsf, 1)
 #undef LBMFVM_RES_WIDE
 
 }  // namespace lbmfvm_dev
