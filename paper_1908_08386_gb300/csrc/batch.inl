@@ -132,20 +132,47 @@ void launch_cav_init(lbmfvm_batch_t *b, int i, const float *u0, const float *v0,
                                              c.grid.bc[2], c.grid.bc[3], Ta, Tb);
 }
 
+// Residual snapshot of cavity i := its current velocity.
 template <class S>
-void launch_cav_residual(lbmfvm_batch_t *b, int i, int update_only) {
+void launch_cav_snapshot(lbmfvm_batch_t *b, int i) {
     lbmfvm_t *h = hnd(b, i);
     int direct;
     StepArgs<S> v = cav_read_view<S>(b, i, direct);
     double *su = reinterpret_cast<double *>(h->base + h->L.snap) + b->cav[i].snap_off;
     double *sv = su + (size_t)b->cav[i].grid.nx * b->cav[i].grid.ny;
-    double *red = reinterpret_cast<double *>(h->base + h->L.red);
     const int blocks = v.ny < kResidualBlocks ? v.ny : kResidualBlocks;
-    residual_kernel<S><<<blocks, 256, 0, h->s>>>(v, direct, su, sv, red, update_only);
-    if (!update_only)
-        residual_finish_kernel<<<1, 32, 0, h->s>>>(red, blocks,
-                                                   reinterpret_cast<double *>(h->base + h->L.cavres) + kCavRes * i, v.err,
-                                                   nullptr);
+    residual_kernel<S><<<blocks, 256, 0, h->s>>>(v, direct, su, sv, nullptr, 1);
+}
+
+// Residual totals of every active cavity of packed grid h into its result
+// table: the list and the partial sums in the staging area.
+template <class S>
+void launch_residuals(lbmfvm_batch_t *b, lbmfvm_t *h, cudaError_t &e) {
+    std::vector<ResidualCav> list;
+    int blocks = 0;
+    for (int i = 0; i < (int)b->cav.size(); i++) {
+        const auto &c = b->cav[i];
+        if (!c.active || hnd(b, i) != h) continue;
+        const int nb = c.grid.ny < kResidualBlocks ? c.grid.ny : kResidualBlocks;
+        list.push_back(ResidualCav{i, blocks, nb, c.steps == 0, (long long)c.snap_off});
+        blocks += nb;
+    }
+    if (list.empty()) return;
+    const int par = h->parity;  // active cavities stand at the grid's parity
+    StepArgs<S> v = args_for<S>(h, par);
+    v.fin = reinterpret_cast<const S *>(h->base + h->L.f[par ^ 1]);
+    unsigned char *stage = h->base + h->L.stage;
+    const size_t head = align_up(list.size() * sizeof(ResidualCav), kAlign);
+    const ResidualCav *dl = reinterpret_cast<const ResidualCav *>(stage);
+    double *partials = reinterpret_cast<double *>(stage + head);
+    const CavityDesc *cavs = reinterpret_cast<const CavityDesc *>(h->base + h->L.cav);
+    e = cudaMemcpyAsync(stage, list.data(), list.size() * sizeof(ResidualCav), cudaMemcpyHostToDevice, h->s);
+    if (e != cudaSuccess) return;
+    residual_cavs_kernel<S><<<blocks, 256, 0, h->s>>>(v, cavs, dl, (int)list.size(),
+                                                      reinterpret_cast<double *>(h->base + h->L.snap), partials);
+    residual_finish_cavs_kernel<<<(unsigned)list.size(), 32, 0, h->s>>>(
+        dl, partials, reinterpret_cast<double *>(h->base + h->L.cavres), kCavRes);
+    e = cudaGetLastError();
 }
 
 template <class S>
@@ -357,7 +384,7 @@ int cav_set_state(lbmfvm_batch_t *b, int i, const float *u, const float *v, cons
     if (e != cudaSuccess) return bfail(b, LBMFVM_ERR_CUDA, "staging the state failed: %s", cudaGetErrorString(e));
     BDISPATCH(h, launch_cav_init, b, i, du, dv, dT);
     b->cav[i].steps = 0;
-    BDISPATCH(h, launch_cav_residual, b, i, 1);  // snapshot := u^0
+    BDISPATCH(h, launch_cav_snapshot, b, i);  // snapshot := u^0
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
     if (e != cudaSuccess) return bfail(b, LBMFVM_ERR_CUDA, "initial state failed: %s", cudaGetErrorString(e));
@@ -579,10 +606,9 @@ int lbmfvm_batch_residuals(lbmfvm_batch_t *b, double *r) {
         lbmfvm_t *h = b->lv[g];
         if (!h) continue;
         if (int e = bcheck_h(b, h, join_in(h))) return e;
-        for (int i = 0; i < n; i++)
-            if (b->cav[i].active && hnd(b, i) == h) BDISPATCH(h, launch_cav_residual, b, i, 0);
+        cudaError_t e = cudaSuccess;
+        BDISPATCH(h, launch_residuals, b, h, e);
         res[g].resize(kCavRes * (size_t)n);
-        cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(res[g].data(), h->base + h->L.cavres, res[g].size() * sizeof(double),
                                 cudaMemcpyDeviceToHost, h->s);

@@ -2180,31 +2180,29 @@ constexpr int kResidualSums = 4;
 // from kHostLocal the local Nusselt numbers.
 constexpr int kHostStatus = 8, kHostLocal = 16;
 
+// One row: adds its sums to v and replaces its snapshot.
 template <class S>
-__global__ void __launch_bounds__(256) residual_kernel(const StepArgs<S> a, int direct, double *su,
-                                                       double *sv, double *partials, int update_only) {
+__device__ __forceinline__ void residual_row(const StepArgs<S> &a, int direct, int y, double *su, double *sv,
+                                             double v[kResidualSums]) {
     using C = typename Compute<S>::type;
-    __shared__ double red[kResidualSums][8];
-    double num = 0.0, den = 0.0, mass = 0.0, cnt = 0.0;
-    for (int y = blockIdx.x; y < a.ny; y += gridDim.x) {
-        for (int x = threadIdx.x; x < a.nx; x += blockDim.x) {
-            const long long k = (long long)y * a.pitch + x;
-            const uint8_t c = decode(a.code[k]);
-            if ((c & 3) != KIND_FLUID) continue;
-            C drho, ux, uy;
-            current_moments<S>(a, direct, x, y, c, drho, ux, uy);
-            const long long i = (long long)y * a.nx + x;
-            const double du = (double)ux - su[i], dv = (double)uy - sv[i];
-            num += du * du + dv * dv;
-            den += (double)ux * (double)ux + (double)uy * (double)uy;
-            mass += (double)drho;
-            cnt += 1.0;
-            su[i] = (double)ux;
-            sv[i] = (double)uy;
-        }
+    for (int x = threadIdx.x; x < a.nx; x += blockDim.x) {
+        const long long k = (long long)y * a.pitch + x;
+        const uint8_t c = decode(a.code[k]);
+        if ((c & 3) != KIND_FLUID) continue;
+        C drho, ux, uy;
+        current_moments<S>(a, direct, x, y, c, drho, ux, uy);
+        const long long i = (long long)y * a.nx + x;
+        const double du = (double)ux - su[i], dv = (double)uy - sv[i];
+        v[0] += du * du + dv * dv;
+        v[1] += (double)ux * (double)ux + (double)uy * (double)uy;
+        v[2] += (double)drho;
+        v[3] += 1.0;
+        su[i] = (double)ux;
+        sv[i] = (double)uy;
     }
-    if (update_only) return;
-    double v[kResidualSums] = {num, den, mass, cnt};
+}
+// A block's sums of v into out[0 .. kResidualSums).
+__device__ __forceinline__ void residual_block_sums(double v[kResidualSums], double (*red)[8], double *out) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int j = 0; j < kResidualSums; j++) {
@@ -2216,14 +2214,11 @@ __global__ void __launch_bounds__(256) residual_kernel(const StepArgs<S> a, int 
     if (threadIdx.x < kResidualSums) {
         double t = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += red[threadIdx.x][w];
-        partials[kResidualSums * blockIdx.x + threadIdx.x] = t;
+        out[threadIdx.x] = t;
     }
 }
-
-// Residual, pass 2: one warp sums the block partials in a fixed order.  host
-// (may be NULL, host-mapped) receives the totals and the device status word.
-static __global__ void residual_finish_kernel(const double *partials, int nblocks, double *out, const int *err,
-                                              double *host) {
+// One warp's totals of nblocks partials, in a fixed order, into out.
+__device__ __forceinline__ void residual_total(const double *partials, int nblocks, double *out) {
     double v[kResidualSums] = {};
     for (int b = threadIdx.x; b < nblocks; b += 32)
 #pragma unroll
@@ -2233,13 +2228,85 @@ static __global__ void residual_finish_kernel(const double *partials, int nblock
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0)
 #pragma unroll
-        for (int j = 0; j < kResidualSums; j++) {
-            out[j] = v[j];
-            if (host) host[j] = v[j];
+        for (int j = 0; j < kResidualSums; j++) out[j] = v[j];
+}
+
+template <class S>
+__global__ void __launch_bounds__(256) residual_kernel(const StepArgs<S> a, int direct, double *su,
+                                                       double *sv, double *partials, int update_only) {
+    __shared__ double red[kResidualSums][8];
+    double v[kResidualSums] = {};
+    for (int y = blockIdx.x; y < a.ny; y += gridDim.x) residual_row<S>(a, direct, y, su, sv, v);
+    if (update_only) return;
+    residual_block_sums(v, red, partials + kResidualSums * blockIdx.x);
+}
+
+// The same over all active cavities of a batch in one launch (two launches per
+// cavity took 0.7-1.1 ms of 64; the passes that hold them got 0.8 ms shorter): one block per row, or per kResidualBlocks-th
+// row of a taller cavity, so that the partial sums and their order are those of
+// the single launches; their totals by residual_finish_cavs_kernel.
+struct ResidualCav {
+    int cav;            // cavity (its descriptor, its slot of the result table)
+    int block0, blocks; // its blocks
+    int direct;         // at step 0
+    long long snap_off; // first node of its residual snapshot
+};
+
+template <class S>
+__global__ void __launch_bounds__(256)
+    residual_cavs_kernel(const StepArgs<S> base, const CavityDesc *__restrict__ cavs,
+                         const ResidualCav *__restrict__ list, int n, double *snap, double *partials) {
+    using C = typename Compute<S>::type;
+    __shared__ double red[kResidualSums][8];
+    int lo = 0, hi = n - 1;  // the last entry whose blocks start at or before this one
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (list[mid].block0 <= (int)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    const ResidualCav e = list[lo];
+    const CavityDesc &cd = cavs[e.cav];
+    StepArgs<S> a = base;
+    const long long off = (long long)cd.y0 * a.pitch + cd.x0;
+    a.fin += off;
+    a.Tin += off;
+    a.code += off;
+    a.nx = cd.nx;
+    a.ny = cd.ny;
+    a.perx = a.pery = 0;
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        if constexpr (std::is_same<C, float>::value) {
+            a.wall_u[s] = cd.wall_uf[s];
+            a.wall_v[s] = cd.wall_vf[s];
+        } else {
+            a.wall_u[s] = C(cd.wall_u[s]);
+            a.wall_v[s] = C(cd.wall_v[s]);
         }
-        if (host) host[kHostStatus] = (double)*err;
+    }
+    double *su = snap + e.snap_off, *sv = su + (size_t)a.nx * a.ny;
+    double v[kResidualSums] = {};
+    for (int y = (int)blockIdx.x - e.block0; y < a.ny; y += e.blocks)
+        residual_row<S>(a, e.direct, y, su, sv, v);
+    residual_block_sums(v, red, partials + kResidualSums * (size_t)blockIdx.x);
+}
+
+static __global__ void residual_finish_cavs_kernel(const ResidualCav *list, const double *partials, double *out,
+                                                   int stride) {
+    const ResidualCav e = list[blockIdx.x];
+    residual_total(partials + kResidualSums * (size_t)e.block0, e.blocks, out + (size_t)stride * e.cav);
+}
+
+// Residual, pass 2: one warp sums the block partials in a fixed order.  host
+// (may be NULL, host-mapped) receives the totals and the device status word.
+static __global__ void residual_finish_kernel(const double *partials, int nblocks, double *out, const int *err,
+                                              double *host) {
+    residual_total(partials, nblocks, out);
+    if (threadIdx.x == 0 && host) {
+        for (int j = 0; j < kResidualSums; j++) host[j] = out[j];
+        host[kHostStatus] = (double)*err;
     }
 }
 

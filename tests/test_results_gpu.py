@@ -69,3 +69,28 @@ def test_batch_fields_into_device_memory():
         out = torch.zeros(4, ny, nx, dtype=torch.float64, device="cuda")
         L._bcheck(L.lib().lbmfvm_batch_fields(b.b, i, *[L._addr(out[j]) for j in range(4)]), b.b)
         assert np.array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("store", ["f32", "f16", "f32x2", "f64"])
+def test_batch_residuals_equal_the_single_handles(store):
+    """One launch over all active cavities (one of more rows than a cavity has
+    blocks, one at step 0, one that has left) against a handle each: the same
+    sums in the same order, so they agree to a few roundings of the FP64 sums."""
+    from paper_1908_08386_gb300 import workloads as WL
+
+    mask = np.zeros((33, 70), np.uint8)
+    mask[10:20, 20:40] = 1
+    cases = [WL.CavityCase(40, 37, 1e4, 0.71, 0.17), WL.CavityCase(70, 33, 1e5, 0.71, 0.17, mask=mask),
+             WL.CavityCase(20, 700, 1e6, 0.71, 0.05), WL.CavityCase(50, 50, 1e5, 7.0, 0.17)]
+    b = L.Batch(cases, store=store, tma_config="default")
+    singles = [L.Cavity(c.nx, c.ny, Ra=c.Ra, Pr=c.Pr, Ma=c.Ma, mask=c.mask, store=store) for c in cases]
+    for n in (7, 12):
+        b.step(n)
+        got = b.residuals()
+        for i, c in enumerate(singles):
+            c.step(n)
+            assert got[i] == pytest.approx(c.residual(), rel=1e-12), i
+    b.set_state(3)  # back to step 0: its snapshot is its state
+    got = b.residuals()
+    assert got[3] == 0.0 and list(got[:3]) == [0.0] * 3
+    b.close()
