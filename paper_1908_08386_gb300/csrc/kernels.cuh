@@ -22,7 +22,9 @@
 //                    written back by TMA bulk stores (walled domains,
 //                    FP32/FP16/BF16 storage);
 //   step_kernel      one block per tile, gathers straight from global memory
-//                    (periodic sides, FP64 storage).
+//                    (periodic sides, finite-difference walls).
+// A third (resident_kernel, resident.cuh) takes many steps of a small grid in one
+// launch with the same arithmetic.
 #pragma once
 
 #include <cuda.h>
@@ -1073,6 +1075,8 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 //           stage's population bytes;
 //   refill  thread 0, once the store of tile k-1 has read its stage, loads
 //           tile k-1+STAGES into it.
+// (With a copying warp, G::PW, that warp stores tile k once its compute warps
+// have written it and refills its stage; a stage marked invalid ends the loop.)
 // A wait that runs out raises a shared abort flag that every thread checks
 // after the barrier, so the block leaves together and a device status word
 // tells the host.

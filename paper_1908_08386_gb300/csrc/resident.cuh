@@ -260,6 +260,8 @@ __device__ __forceinline__ void quad_collide(C g0, C f, C b, int s, C drho, C ux
     if (s == 0) out(0, wq<C>(0), g0, P0, nGu);
 }
 
+constexpr uint64_t kFirstWaitNs = 20 * kWaitLimitNs;
+
 // Arguments of a resident launch: steps from the state a.fin, a.Tin to a.fout,
 // a.Tout (other buffers), on one tile per block.
 template <class S>
@@ -480,7 +482,7 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
     };
     // Reads N packets of the slot of `tag` into base + to[i]; false when a
     // wait ran out.
-    auto read = [&](auto *base, const int *at, const int *to, auto count, uint32_t tag) {
+    auto read = [&](auto *base, const int *at, const int *to, auto count, uint32_t tag, uint64_t limit) {
         constexpr int N = decltype(count)::value;
         const uint64_t *slot = r.mailbox + (size_t)(tag & 1u) * G::PACKETS * WORDS;
         uint64_t t0 = 0;
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             if ((it & 63u) == 63u) {
                 const uint64_t t = tma::globaltimer();
                 if (t0 == 0) t0 = t;
-                else if (t - t0 > kWaitLimitNs) return false;
+                else if (t - t0 > limit) return false;
             }
         }
         return true;
@@ -574,6 +576,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         // Phase B: energy balance (in m sub-steps) and collision.
         const bool last = k + 1 == r.nsteps;
         bool ok = true;
+        // the first exchange also waits for blocks that other work still keeps
+        // off their SMs
+        const uint64_t limit = k == 0 ? kFirstWaitNs : kWaitLimitNs;
         for (int s = 1; s <= m; s++) {
             const C *Tc = T + cb * PL;
             C *To = T + (cb ^ 1) * PL;
@@ -645,7 +650,7 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                 const uint32_t tag = (r.seq0 + (uint32_t)k) * (uint32_t)m + (uint32_t)s;
                 __syncthreads();
                 post_T(To, tag);
-                ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag);
+                ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag, limit);
                 if (!ok) gave_up = 1;
                 __syncthreads();
             }
@@ -687,8 +692,8 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                 if (sf[i] >= 0) mail::post(slot, tid + i * BLOCK, F[sf[i]], tag);
             C *To = T + cb * PL;
             post_T(To, tag_t);
-            ok &= read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag);
-            ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t);
+            ok &= read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag, limit);
+            ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t, limit);
             if (!ok) gave_up = 1;
         }
         __syncthreads();

@@ -152,3 +152,21 @@ def test_resident_run_resumes_from_a_checkpoint(tmp_path):
     for c in (a, b):
         c.step(50)
     same(a, b)
+
+
+def test_resident_launch_beside_other_work_on_the_gpu():
+    """Another stream keeps every SM busy while a resident launch comes up: its
+    blocks start as SMs free up, and the result is the same."""
+    kw = dict(nu=0.03, alpha=0.05, gbeta=1e-4)
+    a, b = L.Cavity(300, 280, **kw), L.Cavity(300, 280, kernel="tma", **kw)
+    m = torch.randn(8192, 8192, device="cuda", dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for _ in range(300):
+            out = m @ m
+    for n in (9, 50, 200):
+        a.step(n)
+    for n in (9, 50, 200):
+        b.step(n)
+    same(a, b)
+    del out
