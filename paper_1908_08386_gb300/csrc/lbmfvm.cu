@@ -991,6 +991,31 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
     return LBMFVM_OK;
 }
 
+// Tiles with box-wall nodes cost a warp of pairs about twice the others (a wall
+// lane takes its warp through the extrapolation and the single-node energy
+// balance), and a block takes every blocks-th tile of the list.  Left in place,
+// the wall columns of some widths fall to the same blocks in every round (600^2
+// FP32: 19 columns, 304 blocks).  They go to the end of the first round (whole
+// rounds of them first), so that each block gets as many as the next and the
+// blocks that take one more tile in the last round have the fewest.  The order
+// of the tiles never changes results.  Us per step, row by row / spread (shape):
+// FP32 600^2 10.8 / 7.6 (4), 400 x 900 9.1 / 7.7 (4), 1024^2 16.0 / 16.3 (4), 4096^2
+// 209 / 206 (5); FP16 530^2 8.9 / 6.9, 1024^2 14.7 / 13.4, 4096^2 167 / 163 (5).
+void spread_wall_tiles(std::vector<TileHeader> &list, int blocks, int tw, int th) {
+    if (blocks < 1 || (int)list.size() <= blocks) return;
+    std::vector<TileHeader> wall, rest;
+    for (const TileHeader &t : list) {
+        const bool w = t.ox == 0 || t.oy == 0 || t.ox + tw >= t.nx || t.oy + th >= t.ny;
+        (w ? wall : rest).push_back(t);
+    }
+    const size_t whole = wall.size() / blocks * blocks, left = wall.size() - whole;
+    const size_t first = std::min(rest.size(), (size_t)blocks - left);
+    list.assign(wall.begin(), wall.begin() + whole);
+    list.insert(list.end(), rest.begin(), rest.begin() + first);
+    list.insert(list.end(), wall.begin() + whole, wall.end());
+    list.insert(list.end(), rest.begin() + first, rest.end());
+}
+
 // Tile lists of the TMA kernel (row by row over every active cavity) and the
 // cavity table, uploaded on the handle's stream: cavities with one energy
 // update per step in the fused list, those with sub-steps in the second list,
@@ -1029,6 +1054,7 @@ int upload_tiles(lbmfvm_t *h, int tw, int th) {
         if ((int)h->split_tiles_at.size() < m) h->split_tiles_at.resize(m, 0);
         for (int sub = 0; sub < m; sub++) h->split_tiles_at[sub] = (int)i + 1;
     }
+    if (store_size(h->prec) <= 4) spread_wall_tiles(fused, h->num_sms * (h->fv_quick ? h->blocks_quick : h->tma_blocks_per_sm), tw, th);
     // count slots (their tile counters cleared), each followed by its headers
     std::vector<TileHeader> all;
     TileHeader slot{};
@@ -1377,10 +1403,11 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
     h->tile_y = opts.tile_y ? opts.tile_y : 8;
     h->use_tma = tma_ok && opts.kernel != LBMFVM_KERNEL_GENERIC;
     // the default shapes are the fastest measured ones: two blocks of 32 x 16
-    // per SM with ring warps for 32-bit storage that fits the L2 (1024^2: 16.0 us
-    // against 16.6), 64 x 16 with a copying warp beyond it (4096^2: 210 against
-    // 213) and for 16-bit storage (1024^2: 14.6 against 15.3; 4096^2: 167.5
-    // against 177.5), two blocks of 32 x 8 per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
+    // per SM with ring warps for 32-bit storage that fits the L2 (600^2: 7.6 us
+    // against 8.8, 900^2 12.7 against 13.7; 1024^2 16.3 against 15.6), 64 x 16 with
+    // a copying warp beyond it (4096^2: 206 against 215) and for 16-bit storage
+    // (1024^2: 13.4 against 14.4; 4096^2: 163 against 171), two blocks of 32 x 8
+    // per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
     // SMs is bound by the latency of one tile, not by the SMs' throughput, and
     // takes the smaller tiles that spread it over more SMs: 64 x 8 (two blocks
     // per SM) for 32- and 16-bit storage, 32 x 8 with ring warps for 64-bit.
