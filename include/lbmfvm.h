@@ -289,6 +289,13 @@ int lbmfvm_step(lbmfvm_t *h, int64_t n);
  * the handle runs the generic kernel, which has no such waits. */
 int lbmfvm_inject_stall(lbmfvm_t *h);
 
+/* Further hooks of this kind, each for the next lbmfvm_step that runs the
+ * kernel it belongs to.  LBMFVM_ERR_ARG if the handle does not run it.
+ *   FAULT_END  tile shape 5 of 32- and 16-bit storage: one warp of block 0
+ *              takes the end of its tiles for a wait that ran out. */
+#define LBMFVM_FAULT_END 1
+int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind);
+
 /* Number of time steps taken since the last set_state. */
 int lbmfvm_step_count(const lbmfvm_t *h, int64_t *steps);
 

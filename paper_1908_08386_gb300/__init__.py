@@ -44,6 +44,8 @@ PRECISIONS = {"f64": LBMFVM_F64, "f32": LBMFVM_F32, "f16": LBMFVM_F16, "bf16": L
 LBMFVM_FV_CENTRAL, LBMFVM_FV_QUICK = 0, 1
 FV_SCHEMES = {"central": LBMFVM_FV_CENTRAL, "quick": LBMFVM_FV_QUICK}
 LBMFVM_FV_SUBSTEPS_AUTO = 0
+# Test hooks of the bounded waits (lbmfvm_inject_fault)
+LBMFVM_FAULT_END = 1
 # Energy solvers
 LBMFVM_ENERGY_FV, LBMFVM_ENERGY_LBM_D2Q5 = 0, 1
 ENERGY = {"fv": LBMFVM_ENERGY_FV, "lbm": LBMFVM_ENERGY_LBM_D2Q5}
@@ -54,7 +56,7 @@ WALLS = {"nee": LBMFVM_WALL_NEE, "fd": LBMFVM_WALL_FD}
 # Every entry point the header declares (checked by the test-suite).
 EXPORTS = (
     "lbmfvm_opts_default", "lbmfvm_workspace_bytes", "lbmfvm_create", "lbmfvm_create_lattice",
-    "lbmfvm_set_state", "lbmfvm_step", "lbmfvm_inject_stall", "lbmfvm_step_count", "lbmfvm_fields", "lbmfvm_fields_f32",
+    "lbmfvm_set_state", "lbmfvm_step", "lbmfvm_inject_stall", "lbmfvm_inject_fault", "lbmfvm_step_count", "lbmfvm_fields", "lbmfvm_fields_f32",
     "lbmfvm_nusselt", "lbmfvm_residual", "lbmfvm_run_to_steady", "lbmfvm_copy_state", "lbmfvm_launch_count", "lbmfvm_kernel_info", "lbmfvm_fv_info", "lbmfvm_params", "lbmfvm_residual_noalloc",
     "lbmfvm_save", "lbmfvm_load", "lbmfvm_checkpoint_info",
     "lbmfvm_destroy", "lbmfvm_last_error", "lbmfvm_batch_create", "lbmfvm_batch_set_state", "lbmfvm_batch_step",
@@ -120,6 +122,7 @@ def lib() -> ctypes.CDLL:
                 "lbmfvm_set_state": (ctypes.c_int, [vp, vp, vp, vp]),
                 "lbmfvm_step": (ctypes.c_int, [vp, i64]),
                 "lbmfvm_inject_stall": (ctypes.c_int, [vp]),
+                "lbmfvm_inject_fault": (ctypes.c_int, [vp, ctypes.c_int32]),
                 "lbmfvm_step_count": (ctypes.c_int, [vp, i64p]),
                 "lbmfvm_fields": (ctypes.c_int, [vp, vp, vp, vp, vp]),
                 "lbmfvm_fields_f32": (ctypes.c_int, [vp, vp, vp, vp, vp]),
@@ -225,6 +228,10 @@ def lbmfvm_step(h, n):
 
 def lbmfvm_inject_stall(h):
     _check(lib().lbmfvm_inject_stall(h), h)
+
+
+def lbmfvm_inject_fault(h, kind):
+    _check(lib().lbmfvm_inject_fault(h, int(kind)), h)
 
 
 def lbmfvm_step_count(h) -> int:

@@ -286,7 +286,7 @@ struct StepArgs {
     C omega, alpha, gbeta, t_ref, fx, fy;
     C wall_u[4], wall_v[4];  // velocity of box walls per side W, E, S, N
     int *err;                // device status word (bounded waits that ran out)
-    int stall;               // test hook: block 0 skips its first staged load
+    int stall;               // test hook of block 0 (kStall*)
     int wall_fd;             // generic kernel: finite-difference velocity-gradient box walls
     C fd_coef;               // their 3 tau (tau w_i / c_s^2 = 3 tau w_i)
 };
@@ -1033,6 +1033,10 @@ constexpr int kTmaConfigFv = 1;
 
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per wait
 constexpr int kErrTimeout = 1;
+// Test hooks of the step kernel, block 0: its first staged load is never issued;
+// its first warp takes the end mark of the block's tiles (copying-warp shape) for
+// a wait that ran out.
+constexpr int kStallLoad = 1, kStallEnd = 2;
 
 namespace tma {
 __device__ __forceinline__ void store_3d(const CUtensorMap *map, const void *src, int x, int y, int z) {
@@ -1179,7 +1183,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                     finish(k);
                 } else {
                     valid[k] = 1;
-                    if (!(a.stall && blockIdx.x == 0 && k == 0)) issue(k, t, origin(t));
+                    if (!(a.stall == kStallLoad && blockIdx.x == 0 && k == 0)) issue(k, t, origin(t));
                     issued++;
                 }
             }
@@ -1211,7 +1215,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
                 if (!ok) {
                     // let the copies already in flight land before the block exits
                     for (int j = k; j < issued; j++)
-                        if (!(a.stall && blockIdx.x == 0 && j == 0))
+                        if (!(a.stall == kStallLoad && blockIdx.x == 0 && j == 0))
                             tma::mbar_wait_bounded(&bars[j % G::STAGES], (uint32_t)(j / G::STAGES) & 1u, kWaitLimitNs / 2);
                     atomicOr(a.err, kErrTimeout);
                     break;
@@ -1239,7 +1243,7 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
         if (blockIdx.x == 0) *ctr_next = 0;
         int k = 0;
         for (; k < G::STAGES && fixed_tile(k) >= 0; k++) {
-            if (!(a.stall && blockIdx.x == 0 && k == 0)) issue(k, fixed_tile(k), origin(fixed_tile(k)));
+            if (!(a.stall == kStallLoad && blockIdx.x == 0 && k == 0)) issue(k, fixed_tile(k), origin(fixed_tile(k)));
             issued = k + 1;
         }
         if (k == G::STAGES) {
@@ -1256,13 +1260,24 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
 
     for (int k = 0; G::PW || k < *known; k++) {
         unsigned char *stg = stage(k);
-        const bool landed = tma::mbar_wait_bounded(&bars[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u, kWaitLimitNs);
+        bool landed = tma::mbar_wait_bounded(&bars[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u, kWaitLimitNs);
+        bool end = false;
+        if constexpr (G::PW) {
+            end = landed && !valid[k % G::STAGES];
+            if (end && a.stall == kStallEnd && blockIdx.x == 0 && tid < 32) landed = end = false;
+        }
         if (!landed) {
             atomicOr(abort_flag, 1);
             atomicOr(a.err, kErrTimeout);
         }
-        if constexpr (G::PW)
-            if (landed && !valid[k % G::STAGES]) break;  // for every thread alike
+        if constexpr (G::PW) {
+            if (end) {
+                // a thread whose wait ran out as the mark came does not know of
+                // the end and goes on to this tile's barrier: meet it there
+                asm volatile("bar.sync 1, %0;" ::"n"(G::CONSUMERS) : "memory");
+                break;
+            }
+        }
         // a stage that never landed has no header: use a harmless one (the
         // block leaves at the next barrier)
         const TileHeader hd = landed ? hdrs[k % G::STAGES] : TileHeader{};

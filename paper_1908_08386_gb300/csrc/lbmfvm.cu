@@ -313,7 +313,7 @@ struct lbmfvm {
     cudaGraphExec_t graph;
     int64_t launches; // step-kernel launches issued (a graph replay counts its kernel nodes)
     bool use_tma;     // persistent TMA kernel (walled domains, 32/16-bit storage)
-    bool stall_next;  // test hook armed by lbmfvm_inject_stall
+    int stall_next;   // test hook of the next ordinary step (kStall*)
     int tma_config;   // tile shape of the TMA kernel
     int num_sms;
     CUtensorMap map_f[2], map_T[2], map_c;
@@ -440,10 +440,10 @@ int fixed_tiles(int ntiles, int blocks, int stages) {
 // its temperature box loaded through map_T.
 template <class S>
 lbmfvm_fv::TmaLaunch<S> tma_args(const lbmfvm_t *h, int cur, TileList list, const CUtensorMap *map_T, int per_sm,
-                                 int stages, cudaStream_t s, bool stall) {
+                                 int stages, cudaStream_t s, int stall) {
     lbmfvm_fv::TmaLaunch<S> l{};
     l.a = args_for<S>(h, cur);
-    l.a.stall = stall ? 1 : 0;
+    l.a.stall = stall;
     l.cavs = reinterpret_cast<const CavityDesc *>(h->base + h->L.cav);
     // the count sits at a fixed address in front of the list, so that a
     // captured graph reads the current count after the list has changed
@@ -485,7 +485,7 @@ void launch_split(const lbmfvm_t *h, int cur, cudaStream_t s) {
         lbmfvm_fv::launch_substep<C>(h->fv_quick, T0, X, Y, U, V, h->base + h->L.code, h->base + h->L.fflags,
                                      h->L.pitch, h->grid.nx, h->grid.ny, tiles, h->split_tiles_at[sub - 1],
                                      h->tile_w, h->tile_h, sub, s);
-    lbmfvm_fv::launch_given<S>(tma_args<S>(h, cur, list, &h->map_TX, h->blocks_given, G::STAGES, s, false));
+    lbmfvm_fv::launch_given<S>(tma_args<S>(h, cur, list, &h->map_TX, h->blocks_given, G::STAGES, s, 0));
 }
 
 Grid2Args grid2_args(const lbmfvm_t *h) {
@@ -528,11 +528,11 @@ void launch_grid2(const lbmfvm_t *h, int cur, cudaStream_t s, bool fv_now) {
         const C *Tdir = reinterpret_cast<const C *>(h->base + h->L.T[cur]);
         grid2_nodes_kernel<C><<<gn, b, 0, s>>>(g, h->base + h->L.code, Tdir, Tn, Tc, X, nullptr, nullptr);
     }
-    lbmfvm_fv::launch_given<S>(tma_args<S>(h, cur, list, &h->map_TX, h->blocks_given, G::STAGES, s, false));
+    lbmfvm_fv::launch_given<S>(tma_args<S>(h, cur, list, &h->map_TX, h->blocks_given, G::STAGES, s, 0));
 }
 
 template <class S>
-void launch_step_tma(const lbmfvm_t *h, int cur, cudaStream_t s, bool stall, bool fv_now) {
+void launch_step_tma(const lbmfvm_t *h, int cur, cudaStream_t s, int stall, bool fv_now) {
     if (h->fv_quick) {
         using G = typename TmaConfig<S, kTmaConfigFv>::G;
         lbmfvm_fv::launch_quick<S>(
@@ -546,7 +546,7 @@ void launch_step_tma(const lbmfvm_t *h, int cur, cudaStream_t s, bool stall, boo
 }
 
 template <class S>
-void launch_step(const lbmfvm_t *h, int cur, cudaStream_t s, bool stall, bool fv_now) {
+void launch_step(const lbmfvm_t *h, int cur, cudaStream_t s, int stall, bool fv_now) {
     if (h->use_tma) {
         launch_step_tma<S>(h, cur, s, stall, fv_now);
         return;
@@ -578,7 +578,7 @@ void launch_lbm5(const lbmfvm_t *h, int cur, cudaStream_t s) {
 
 // One coupled step at parity cur; fv_now: grid setting 2 takes its coarse
 // energy step in this one.
-void launch_one(const lbmfvm_t *h, int cur, cudaStream_t s, bool stall = false, bool fv_now = true) {
+void launch_one(const lbmfvm_t *h, int cur, cudaStream_t s, int stall = 0, bool fv_now = true) {
     if (h->energy == LBMFVM_ENERGY_LBM_D2Q5) {
         switch (h->prec) {
             case LBMFVM_F64: launch_lbm5<double>(h, cur, s); break;
@@ -613,7 +613,7 @@ int build_graph(lbmfvm_t *h) {
     CU(h, cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal));
     // a graph starts at a step count that is a multiple of the coarse step
     // interval (which divides kGraphSteps), so its coarse steps sit at fixed places
-    for (int i = 0; i < kGraphSteps; i++) launch_one(h, i & 1, h->s, false, (i + 1) % h->fv_every == 0);
+    for (int i = 0; i < kGraphSteps; i++) launch_one(h, i & 1, h->s, 0, (i + 1) % h->fv_every == 0);
     cudaError_t e = cudaStreamEndCapture(h->s, &g);
     if (e != cudaSuccess) return fail(h, LBMFVM_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
     e = cudaGraphInstantiate(&h->graph, g, 0);
@@ -1625,7 +1625,7 @@ int step_impl(lbmfvm_t *h, int64_t n) {
             h->launches += kGraphSteps;
         } else {
             launch_one(h, h->parity, h->s, h->stall_next, (h->steps + 1) % h->fv_every == 0);
-            h->stall_next = false;
+            h->stall_next = 0;
             CU(h, cudaGetLastError());
             h->parity ^= 1;
             n--;
@@ -1730,8 +1730,20 @@ int lbmfvm_fv_info(const lbmfvm_t *h, int32_t *scheme, int32_t *substeps) {
 int lbmfvm_inject_stall(lbmfvm_t *h) {
     if (!h) return fail_thread(LBMFVM_ERR_ARG, "handle is NULL");
     if (!h->use_tma) return fail(h, LBMFVM_ERR_ARG, "the generic step kernel has no staged loads to stall");
-    h->stall_next = true;
+    h->stall_next = kStallLoad;
     return LBMFVM_OK;
+}
+
+int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind) {
+    if (!h) return fail_thread(LBMFVM_ERR_ARG, "handle is NULL");
+    switch (kind) {
+        case LBMFVM_FAULT_END:
+            if (!h->use_tma || h->tma_config != 5 || store_size(h->prec) > 4)
+                return fail(h, LBMFVM_ERR_ARG, "only tile shape 5 of 32- and 16-bit storage has an end mark");
+            h->stall_next = kStallEnd;
+            return LBMFVM_OK;
+    }
+    return fail(h, LBMFVM_ERR_ARG, "kind = %d is not a LBMFVM_FAULT_* value", kind);
 }
 
 int lbmfvm_step_count(const lbmfvm_t *h, int64_t *steps) {

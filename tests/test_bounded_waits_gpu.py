@@ -1,0 +1,68 @@
+"""Device-side waits that run out (GPU): the kernel gives up, the next
+synchronising call reports it, and the handle and the context stay usable.
+Nothing here faults or hangs: the hooks make a thread take a wait for one that
+ran out, or leave out what it waits for."""
+
+import numpy as np
+import pytest
+
+import paper_1908_08386_gb300 as L
+from paper_1908_08386_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+KW = dict(nu=0.03, alpha=0.05, gbeta=1e-4)
+
+
+def state(nx, ny, seed):
+    u, v = WL.random_velocity(ny, nx, seed, 0.01)
+    T = WL.random_temperature(ny, nx, seed + 1)
+    return [a.astype(np.float32) for a in (u, v, T)]
+
+
+def reports_and_recovers(c, ref, steps):
+    """The armed call's failure is reported once; from a new state the handle
+    computes what an undisturbed one does."""
+    with pytest.raises(L.LbmfvmError) as e:
+        c.residual()
+    assert e.value.code == L.LBMFVM_ERR_TIMEOUT
+    for h in (c, ref):
+        h.set_state(*state(c.nx, c.ny, 5))
+        h.step(steps)
+    assert np.array_equal(np.stack(c.fields()), np.stack(ref.fields()))
+    c.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("store", ["f32", "f16"])
+# fewer tiles than blocks' stages, several rounds of tiles, tiles drawn from the counter
+@pytest.mark.parametrize("nx,ny", [(100, 60), (900, 700), (2000, 1500)])
+def test_a_timeout_beside_the_end_mark_leaves_the_block(nx, ny, store):
+    """Copying-warp shape: some threads of a block see the end of its tiles,
+    others a wait that ran out; all of them leave."""
+    kw = dict(KW, store=store, kernel="tma", tma_config=5)
+    c = L.Cavity(nx, ny, **kw)
+    L.lbmfvm_inject_fault(c.h, L.LBMFVM_FAULT_END)
+    c.step(1)
+    reports_and_recovers(c, L.Cavity(nx, ny, **kw), 9)
+
+
+@pytest.mark.parametrize("nx,ny", [(100, 60), (900, 700)])
+def test_a_lost_load_of_the_copying_warp_shape(nx, ny):
+    kw = dict(KW, kernel="tma", tma_config=5)
+    c = L.Cavity(nx, ny, **kw)
+    L.lbmfvm_inject_stall(c.h)
+    c.step(1)
+    reports_and_recovers(c, L.Cavity(nx, ny, **kw), 9)
+
+
+def test_hooks_of_kernels_that_are_not_in_use_are_refused():
+    for kw in (dict(tma_config=4, kernel="tma"), dict(store="f64"), dict(kernel="generic")):
+        c = L.Cavity(40, 40, **dict(KW, **kw))
+        with pytest.raises(L.LbmfvmError) as e:
+            L.lbmfvm_inject_fault(c.h, L.LBMFVM_FAULT_END)
+        assert e.value.code == L.LBMFVM_ERR_ARG
+        with pytest.raises(L.LbmfvmError) as e:
+            L.lbmfvm_inject_fault(c.h, 99)
+        assert e.value.code == L.LBMFVM_ERR_ARG
+        c.close()
