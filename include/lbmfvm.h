@@ -292,8 +292,15 @@ int lbmfvm_inject_stall(lbmfvm_t *h);
 /* Further hooks of this kind, each for the next lbmfvm_step that runs the
  * kernel it belongs to.  LBMFVM_ERR_ARG if the handle does not run it.
  *   FAULT_END  tile shape 5 of 32- and 16-bit storage: one warp of block 0
- *              takes the end of its tiles for a wait that ran out. */
+ *              takes the end of its tiles for a wait that ran out.
+ *   FAULT_POST, FAULT_SUBPOST  a resident launch (LBMFVM_KERNEL_AUTO) of two or
+ *              more tiles: block 0 leaves out the border values of one step, or
+ *              of the last step's first energy sub-step.  Its neighbours' waits
+ *              give up after about one second and the launch ends.  A single
+ *              cavity's lbmfvm_step takes up to 65536 steps per launch. */
 #define LBMFVM_FAULT_END 1
+#define LBMFVM_FAULT_POST 2
+#define LBMFVM_FAULT_SUBPOST 3
 int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind);
 
 /* Number of time steps taken since the last set_state. */

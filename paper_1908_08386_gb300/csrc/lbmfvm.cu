@@ -314,6 +314,7 @@ struct lbmfvm {
     int64_t launches; // step-kernel launches issued (a graph replay counts its kernel nodes)
     bool use_tma;     // persistent TMA kernel (walled domains, 32/16-bit storage)
     int stall_next;   // test hook of the next ordinary step (kStall*)
+    int fault_next;   // test hook of the next resident launch (LBMFVM_FAULT_*)
     int tma_config;   // tile shape of the TMA kernel
     int num_sms;
     CUtensorMap map_f[2], map_T[2], map_c;
@@ -1572,6 +1573,9 @@ int launch_resident(lbmfvm_t *h, int n) {
     r.tile_h = h->tile_h;
     r.ctr[0] = reinterpret_cast<int *>(h->base + list_fused(h).slot) + 1;
     r.ctr[1] = reinterpret_cast<int *>(h->base + list_split(h).slot) + 1;
+    r.hold_step = h->fault_next == LBMFVM_FAULT_POST ? n / 2 : h->fault_next == LBMFVM_FAULT_SUBPOST ? n - 1 : -1;
+    r.hold_sub = h->fault_next == LBMFVM_FAULT_POST ? h->fv_sub : 1;
+    h->fault_next = 0;
     int dev = 0;
     CU(h, cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(h, LBMFVM_ERR_CUDA, "device %d", dev);
@@ -1741,6 +1745,14 @@ int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind) {
             if (!h->use_tma || h->tma_config != 5 || store_size(h->prec) > 4)
                 return fail(h, LBMFVM_ERR_ARG, "only tile shape 5 of 32- and 16-bit storage has an end mark");
             h->stall_next = kStallEnd;
+            return LBMFVM_OK;
+        case LBMFVM_FAULT_SUBPOST:
+            if (h->fv_sub < 2) return fail(h, LBMFVM_ERR_ARG, "the handle takes no energy sub-steps");
+            [[fallthrough]];
+        case LBMFVM_FAULT_POST:
+            if (h->res_shape < 0 || h->res_tiles < 2)
+                return fail(h, LBMFVM_ERR_ARG, "the handle has no resident launches with an exchange");
+            h->fault_next = kind;
             return LBMFVM_OK;
     }
     return fail(h, LBMFVM_ERR_ARG, "kind = %d is not a LBMFVM_FAULT_* value", kind);

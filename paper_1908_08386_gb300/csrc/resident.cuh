@@ -276,6 +276,9 @@ struct ResArgs {
     int quick;                // QUICK face values (general form)
     int tile_w, tile_h;       // tiles of the step kernel
     int *ctr[2];              // tile counters of the step kernel's lists, cleared for the next launch
+    // test hook: block 0 leaves out what it posts in sub-step hold_sub (of m) of
+    // step hold_step (-1: none)
+    int hold_step, hold_sub;
 };
 
 // GENERAL: QUICK face values and energy sub-steps; else the central update,
@@ -515,6 +518,8 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         for (int q = 0; q < 9; q++) g[q] = ld(p + q * PL - cy(q) * FW - cx(q));
     };
 
+    auto held = [&](int k, int s) { return r.hold_step == k && r.hold_sub == s && blockIdx.x == 0; };
+
     int cb = 0;  // temperature plane of the current step
     for (int k = 0; k < r.nsteps; k++) {
         // Phase A: moments of the own nodes (kept in registers) and of the ring.
@@ -649,10 +654,15 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             if (s < m) {
                 const uint32_t tag = (r.seq0 + (uint32_t)k) * (uint32_t)m + (uint32_t)s;
                 __syncthreads();
-                post_T(To, tag);
-                ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag, limit);
+                if (!held(k, s)) post_T(To, tag);
+                ok = read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag, limit);
                 if (!ok) gave_up = 1;
                 __syncthreads();
+                // (the last step makes no other exchange that would report it)
+                if (gave_up) {
+                    if (!ok) atomicOr(r.a.err, kErrTimeout);
+                    return;
+                }
             }
         }
         if (computes) {
@@ -687,13 +697,15 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             const uint32_t tag = r.seq0 + (uint32_t)k + 1u;
             const uint32_t tag_t = (r.seq0 + (uint32_t)k) * (uint32_t)m + (uint32_t)m;
             uint64_t *slot = own + (size_t)(tag & 1u) * G::PACKETS * WORDS;
-#pragma unroll
-            for (int i = 0; i < NSF; i++)
-                if (sf[i] >= 0) mail::post(slot, tid + i * BLOCK, F[sf[i]], tag);
             C *To = T + cb * PL;
-            post_T(To, tag_t);
-            ok &= read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag, limit);
-            ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t, limit);
+            if (!held(k, m)) {
+#pragma unroll
+                for (int i = 0; i < NSF; i++)
+                    if (sf[i] >= 0) mail::post(slot, tid + i * BLOCK, F[sf[i]], tag);
+                post_T(To, tag_t);
+            }
+            ok = read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag, limit) &&
+                 read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t, limit);
             if (!ok) gave_up = 1;
         }
         __syncthreads();

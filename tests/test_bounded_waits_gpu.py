@@ -56,6 +56,19 @@ def test_a_lost_load_of_the_copying_warp_shape(nx, ny):
     reports_and_recovers(c, L.Cavity(nx, ny, **kw), 9)
 
 
+@pytest.mark.parametrize("store", ["f32", "f16", "f32x2", "f64"])
+@pytest.mark.parametrize("fault,m", [("POST", 1), ("POST", 3), ("SUBPOST", 2), ("SUBPOST", 3)])
+def test_a_border_that_is_never_posted_is_reported(store, fault, m):
+    """Resident launches: the exchange of a step, of a step with energy
+    sub-steps, and between the sub-steps of the last step, which no later
+    exchange follows."""
+    kw = dict(KW, alpha=0.05 * m, store=store, fv_substeps=m)
+    c = L.Cavity(70, 90, **kw)
+    L.lbmfvm_inject_fault(c.h, getattr(L, "LBMFVM_FAULT_" + fault))
+    c.step(60)
+    reports_and_recovers(c, L.Cavity(70, 90, **dict(kw, kernel="tma")), 33)
+
+
 def test_hooks_of_kernels_that_are_not_in_use_are_refused():
     for kw in (dict(tma_config=4, kernel="tma"), dict(store="f64"), dict(kernel="generic")):
         c = L.Cavity(40, 40, **dict(KW, **kw))
@@ -64,5 +77,8 @@ def test_hooks_of_kernels_that_are_not_in_use_are_refused():
         assert e.value.code == L.LBMFVM_ERR_ARG
         with pytest.raises(L.LbmfvmError) as e:
             L.lbmfvm_inject_fault(c.h, 99)
+        assert e.value.code == L.LBMFVM_ERR_ARG
+        with pytest.raises(L.LbmfvmError) as e:
+            L.lbmfvm_inject_fault(c.h, L.LBMFVM_FAULT_SUBPOST)
         assert e.value.code == L.LBMFVM_ERR_ARG
         c.close()
