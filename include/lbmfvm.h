@@ -83,7 +83,10 @@ extern "C" {
  * to the library too (tma_config TMA_DEFAULT or TMA_AUTOTUNE), grids and batches
  * whose tiles fit the SMs one per block (up to about 300,000 nodes in FP32, 75,000
  * in 64-bit types) run all but the last of eight or more steps of a call in one
- * launch that keeps the state on the chip, with the same results.  Such launches
+ * launch that keeps the state on the chip, with the same results.  The blocks of
+ * such a launch wait for one another: other work that keeps some of them off
+ * their SMs for more than two minutes makes the call fail with
+ * LBMFVM_ERR_TIMEOUT.  Such launches
  * of one process go one after another on a device, and are not taken while the
  * stream is being captured. */
 #define LBMFVM_KERNEL_AUTO 0
@@ -297,10 +300,13 @@ int lbmfvm_inject_stall(lbmfvm_t *h);
  *              more tiles: block 0 leaves out the border values of one step, or
  *              of the last step's first energy sub-step.  Its neighbours' waits
  *              give up after about one second and the launch ends.  A single
- *              cavity's lbmfvm_step takes up to 65536 steps per launch. */
+ *              cavity's lbmfvm_step takes up to 65536 steps per launch.
+ *   FAULT_LATE  a resident launch whose block 0 starts 0.25 s late and whose
+ *              waits give up after 0.02 s once all blocks run: not a failure. */
 #define LBMFVM_FAULT_END 1
 #define LBMFVM_FAULT_POST 2
 #define LBMFVM_FAULT_SUBPOST 3
+#define LBMFVM_FAULT_LATE 4
 int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind);
 
 /* Number of time steps taken since the last set_state. */

@@ -1575,6 +1575,11 @@ int launch_resident(lbmfvm_t *h, int n) {
     r.ctr[1] = reinterpret_cast<int *>(h->base + list_split(h).slot) + 1;
     r.hold_step = h->fault_next == LBMFVM_FAULT_POST ? n / 2 : h->fault_next == LBMFVM_FAULT_SUBPOST ? n - 1 : -1;
     r.hold_sub = h->fault_next == LBMFVM_FAULT_POST ? h->fv_sub : 1;
+    r.wait_ns = kWaitLimitNs;
+    if (h->fault_next == LBMFVM_FAULT_LATE) {
+        r.wait_ns = kWaitLimitNs / 50;
+        r.late_ns = kWaitLimitNs / 4;
+    }
     h->fault_next = 0;
     int dev = 0;
     CU(h, cudaGetDevice(&dev));
@@ -1750,6 +1755,7 @@ int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind) {
             if (h->fv_sub < 2) return fail(h, LBMFVM_ERR_ARG, "the handle takes no energy sub-steps");
             [[fallthrough]];
         case LBMFVM_FAULT_POST:
+        case LBMFVM_FAULT_LATE:
             if (h->res_shape < 0 || h->res_tiles < 2)
                 return fail(h, LBMFVM_ERR_ARG, "the handle has no resident launches with an exchange");
             h->fault_next = kind;

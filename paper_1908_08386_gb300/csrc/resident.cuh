@@ -260,7 +260,9 @@ __device__ __forceinline__ void quad_collide(C g0, C f, C b, int s, C drho, C ux
     if (s == 0) out(0, wq<C>(0), g0, P0, nGu);
 }
 
-constexpr uint64_t kFirstWaitNs = 20 * kWaitLimitNs;
+// Limit of the waits in which a block may still be kept off its SM by other work
+// (the blocks that run wait meanwhile, as the whole launch would for SMs).
+constexpr uint64_t kStartWaitNs = 120 * kWaitLimitNs;
 
 // Arguments of a resident launch: steps from the state a.fin, a.Tin to a.fout,
 // a.Tout (other buffers), on one tile per block.
@@ -279,6 +281,8 @@ struct ResArgs {
     // test hook: block 0 leaves out what it posts in sub-step hold_sub (of m) of
     // step hold_step (-1: none)
     int hold_step, hold_sub;
+    uint64_t late_ns;         // test hook: block 0 starts this much later
+    uint64_t wait_ns;         // limit of a wait once every block runs
 };
 
 // GENERAL: QUICK face values and energy sub-steps; else the central update,
@@ -321,6 +325,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         const int x = ox + lx, y = oy + ly;
         return x == 0 ? 0 : (x == cnx - 1 ? 1 : (y == 0 ? 2 : 3));
     };
+
+    if (r.late_ns && blockIdx.x == 0)
+        for (const uint64_t t0 = tma::globaltimer(); tma::globaltimer() - t0 < r.late_ns;) __nanosleep(1000);
 
     // The staged box of the state to start from (nothing outside the cavity).
     for (int i = tid; i < PL; i += BLOCK) {
@@ -425,7 +432,8 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
     // a packet index of the neighbour's mailbox (-1: nothing there).
     constexpr int NSF = G::NSF, NRF = G::NRF, NST = G::NST, NRD = G::NRD;
     int sf[NSF], rf_at[NRF], rf_to[NRF], rt_at[NRD], rt_to[NRD];
-    const int ntx = (cnx + TW - 1) / TW;
+    const int ntx = (cnx + TW - 1) / TW, nty = (cny + TH - 1) / TH;
+    const int reach = ntx > nty ? ntx : nty;  // steps by which every block of the cavity has been waited for
     auto packet_of = [&](int lx, int ly, auto index) {  // of node (lx, ly) outside the tile
         if (!in_cavity(lx, ly)) return -1;
         const int dx = lx < 0 ? -1 : (lx >= TW ? 1 : 0), dy = ly < 0 ? -1 : (ly >= TH ? 1 : 0);
@@ -581,9 +589,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         // Phase B: energy balance (in m sub-steps) and collision.
         const bool last = k + 1 == r.nsteps;
         bool ok = true;
-        // the first exchange also waits for blocks that other work still keeps
-        // off their SMs
-        const uint64_t limit = k == 0 ? kFirstWaitNs : kWaitLimitNs;
+        // An exchange is between neighbours: a block that other work still keeps
+        // off its SM holds up those d tiles away in exchange d - 1.
+        const uint64_t limit = k < reach ? kStartWaitNs : r.wait_ns;
         for (int s = 1; s <= m; s++) {
             const C *Tc = T + cb * PL;
             C *To = T + (cb ^ 1) * PL;

@@ -69,6 +69,26 @@ def test_a_border_that_is_never_posted_is_reported(store, fault, m):
     reports_and_recovers(c, L.Cavity(70, 90, **dict(kw, kernel="tma")), 33)
 
 
+# two tiles; four and more across in x, in y and in both; shapes of one and of several nodes per thread
+@pytest.mark.parametrize("nx,ny,store,m", [(20, 8, "f32", 1), (120, 20, "f32", 1), (20, 120, "f32", 3), (300, 280, "f32", 1),
+                                           (300, 280, "f16", 2), (90, 60, "f32x2", 2), (60, 60, "f64", 1)])
+def test_a_block_that_starts_late_is_waited_for(nx, ny, store, m):
+    """A resident launch whose first block is kept off its SM for longer than
+    the limit of a running exchange: every block waits for it, however far away."""
+    kw = dict(KW, alpha=0.05 * m, store=store, fv_substeps=m)
+    c, ref = L.Cavity(nx, ny, **kw), L.Cavity(nx, ny, kernel="tma", **kw)
+    for h in (c, ref):
+        h.set_state(*state(nx, ny, 9))
+    L.lbmfvm_inject_fault(c.h, L.LBMFVM_FAULT_LATE)
+    for n in (60, 9):
+        c.step(n)
+        ref.step(n)
+    assert c.residual() == ref.residual()
+    assert np.array_equal(np.stack(c.fields()), np.stack(ref.fields()))
+    c.close()
+    ref.close()
+
+
 def test_hooks_of_kernels_that_are_not_in_use_are_refused():
     for kw in (dict(tma_config=4, kernel="tma"), dict(store="f64"), dict(kernel="generic")):
         c = L.Cavity(40, 40, **dict(KW, **kw))
