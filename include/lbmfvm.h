@@ -296,11 +296,11 @@ int lbmfvm_inject_stall(lbmfvm_t *h);
  * kernel it belongs to.  LBMFVM_ERR_ARG if the handle does not run it.
  *   FAULT_END  tile shape 5 of 32- and 16-bit storage: one warp of block 0
  *              takes the end of its tiles for a wait that ran out.
- *   FAULT_POST, FAULT_SUBPOST  a resident launch (LBMFVM_KERNEL_AUTO) of two or
- *              more tiles: block 0 leaves out the border values of one step, or
- *              of the last step's first energy sub-step.  Its neighbours' waits
- *              give up after about one second and the launch ends.  A single
- *              cavity's lbmfvm_step takes up to 65536 steps per launch.
+ *   FAULT_POST  a resident launch (LBMFVM_KERNEL_AUTO) of two or more tiles:
+ *              block 0's border values never reach its neighbours.  Their waits
+ *              give up after about one second and the launch ends.
+ *   FAULT_SUBPOST  the same in a launch of one step with energy sub-steps, whose
+ *              only exchanges lie between the sub-steps.
  *   FAULT_LATE  a resident launch whose block 0 starts 0.25 s late and whose
  *              waits give up after 0.02 s once all blocks run: not a failure. */
 #define LBMFVM_FAULT_END 1

@@ -1573,12 +1573,18 @@ int launch_resident(lbmfvm_t *h, int n) {
     r.tile_h = h->tile_h;
     r.ctr[0] = reinterpret_cast<int *>(h->base + list_fused(h).slot) + 1;
     r.ctr[1] = reinterpret_cast<int *>(h->base + list_split(h).slot) + 1;
-    r.hold_step = h->fault_next == LBMFVM_FAULT_POST ? n / 2 : h->fault_next == LBMFVM_FAULT_SUBPOST ? n - 1 : -1;
-    r.hold_sub = h->fault_next == LBMFVM_FAULT_POST ? h->fv_sub : 1;
+    r.start_ns = kStartWaitNs;
     r.wait_ns = kWaitLimitNs;
-    if (h->fault_next == LBMFVM_FAULT_LATE) {
-        r.wait_ns = kWaitLimitNs / 50;
-        r.late_ns = kWaitLimitNs / 4;
+    switch (h->fault_next) {
+        case LBMFVM_FAULT_POST:
+        case LBMFVM_FAULT_SUBPOST:
+            r.spoil = 0x80000000u;  // (a tag's lowest bit chooses the slot)
+            r.start_ns = kWaitLimitNs;
+            break;
+        case LBMFVM_FAULT_LATE:
+            r.late_ns = kWaitLimitNs / 4;
+            r.wait_ns = kWaitLimitNs / 50;
+            break;
     }
     h->fault_next = 0;
     int dev = 0;
@@ -1613,7 +1619,8 @@ int run_resident(lbmfvm_t *h, int n) {
 int step_impl(lbmfvm_t *h, int64_t n) {
     if (resident_steps(h, n)) {
         while (n > 1) {
-            const int k = (int)std::min<int64_t>(n - 1, kResidentSteps);
+            int k = (int)std::min<int64_t>(n - 1, kResidentSteps);
+            if (h->fault_next == LBMFVM_FAULT_SUBPOST) k = 1;
             if (int r = run_resident(h, k)) return r;
             n -= k;
         }

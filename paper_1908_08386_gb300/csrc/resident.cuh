@@ -260,8 +260,7 @@ __device__ __forceinline__ void quad_collide(C g0, C f, C b, int s, C drho, C ux
     if (s == 0) out(0, wq<C>(0), g0, P0, nGu);
 }
 
-// Limit of the waits in which a block may still be kept off its SM by other work
-// (the blocks that run wait meanwhile, as the whole launch would for SMs).
+// Limit of the waits in which a block may still be kept off its SM by other work.
 constexpr uint64_t kStartWaitNs = 120 * kWaitLimitNs;
 
 // Arguments of a resident launch: steps from the state a.fin, a.Tin to a.fout,
@@ -278,11 +277,11 @@ struct ResArgs {
     int quick;                // QUICK face values (general form)
     int tile_w, tile_h;       // tiles of the step kernel
     int *ctr[2];              // tile counters of the step kernel's lists, cleared for the next launch
-    // test hook: block 0 leaves out what it posts in sub-step hold_sub (of m) of
-    // step hold_step (-1: none)
-    int hold_step, hold_sub;
+    uint32_t spoil;           // test hook: block 0's border values carry tags that nobody waits for
     uint64_t late_ns;         // test hook: block 0 starts this much later
-    uint64_t wait_ns;         // limit of a wait once every block runs
+    // limits of a wait: while a block may still be kept off its SM by other work,
+    // and once every block runs
+    uint64_t start_ns, wait_ns;
 };
 
 // GENERAL: QUICK face values and energy sub-steps; else the central update,
@@ -491,9 +490,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             mail::post(slot, G::SF + e, Tn[fi(x, y)], tag);
         }
     };
-    // Reads N packets of the slot of `tag` into base + to[i]; false when a
-    // wait ran out.
-    auto read = [&](auto *base, const int *at, const int *to, auto count, uint32_t tag, uint64_t limit) {
+    // Reads N packets of the slot of `tag` into base + to[i] in step k; false when
+    // a wait ran out.
+    auto read = [&](auto *base, const int *at, const int *to, auto count, uint32_t tag, int k) {
         constexpr int N = decltype(count)::value;
         const uint64_t *slot = r.mailbox + (size_t)(tag & 1u) * G::PACKETS * WORDS;
         uint64_t t0 = 0;
@@ -515,7 +514,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             if ((it & 63u) == 63u) {
                 const uint64_t t = tma::globaltimer();
                 if (t0 == 0) t0 = t;
-                else if (t - t0 > limit) return false;
+                // an exchange is between neighbours: a block that starts late
+                // holds up those d tiles away in exchange d - 1
+                else if (t - t0 > (k < reach ? r.start_ns : r.wait_ns)) return false;
             }
         }
         return true;
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         for (int q = 0; q < 9; q++) g[q] = ld(p + q * PL - cy(q) * FW - cx(q));
     };
 
-    auto held = [&](int k, int s) { return r.hold_step == k && r.hold_sub == s && blockIdx.x == 0; };
+    const uint32_t spoil = blockIdx.x == 0 ? r.spoil : 0u;
 
     int cb = 0;  // temperature plane of the current step
     for (int k = 0; k < r.nsteps; k++) {
@@ -589,9 +590,6 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
         // Phase B: energy balance (in m sub-steps) and collision.
         const bool last = k + 1 == r.nsteps;
         bool ok = true;
-        // An exchange is between neighbours: a block that other work still keeps
-        // off its SM holds up those d tiles away in exchange d - 1.
-        const uint64_t limit = k < reach ? kStartWaitNs : r.wait_ns;
         for (int s = 1; s <= m; s++) {
             const C *Tc = T + cb * PL;
             C *To = T + (cb ^ 1) * PL;
@@ -662,8 +660,8 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             if (s < m) {
                 const uint32_t tag = (r.seq0 + (uint32_t)k) * (uint32_t)m + (uint32_t)s;
                 __syncthreads();
-                if (!held(k, s)) post_T(To, tag);
-                ok = read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag, limit);
+                post_T(To, tag ^ spoil);
+                ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag, k);
                 if (!ok) gave_up = 1;
                 __syncthreads();
                 // (the last step makes no other exchange that would report it)
@@ -706,14 +704,13 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
             const uint32_t tag_t = (r.seq0 + (uint32_t)k) * (uint32_t)m + (uint32_t)m;
             uint64_t *slot = own + (size_t)(tag & 1u) * G::PACKETS * WORDS;
             C *To = T + cb * PL;
-            if (!held(k, m)) {
 #pragma unroll
-                for (int i = 0; i < NSF; i++)
-                    if (sf[i] >= 0) mail::post(slot, tid + i * BLOCK, F[sf[i]], tag);
-                post_T(To, tag_t);
-            }
-            ok = read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag, limit) &&
-                 read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t, limit);
+            for (int i = 0; i < NSF; i++)
+                if (sf[i] >= 0) mail::post(slot, tid + i * BLOCK, F[sf[i]], tag ^ spoil);
+            post_T(To, tag_t ^ spoil);
+            // (both, one after the other's success or not: their first loads overlap)
+            ok &= read(F, rf_at, rf_to, std::integral_constant<int, NRF>{}, tag, k);
+            ok &= read(To, rt_at, rt_to, std::integral_constant<int, NRD>{}, tag_t, k);
             if (!ok) gave_up = 1;
         }
         __syncthreads();
