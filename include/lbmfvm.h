@@ -86,8 +86,9 @@ extern "C" {
  * launch that keeps the state on the chip, with the same results.  The blocks of
  * such a launch wait for one another: other work that keeps some of them off
  * their SMs for more than two minutes makes the call fail with
- * LBMFVM_ERR_TIMEOUT.  Such launches
- * of one process go one after another on a device, and are not taken while the
+ * LBMFVM_ERR_TIMEOUT.  A call
+ * takes its steps one per launch where the device has no room for such a launch
+ * beside those of handles on other streams that are still in flight, and while the
  * stream is being captured. */
 #define LBMFVM_KERNEL_AUTO 0
 #define LBMFVM_KERNEL_GENERIC 1
@@ -302,11 +303,14 @@ int lbmfvm_inject_stall(lbmfvm_t *h);
  *   FAULT_SUBPOST  the same in a launch of one step with energy sub-steps, whose
  *              only exchanges lie between the sub-steps.
  *   FAULT_LATE  a resident launch whose block 0 starts 0.25 s late and whose
- *              waits give up after 0.02 s once all blocks run: not a failure. */
+ *              waits give up after 0.02 s once all blocks run: not a failure.
+ *   FAULT_REFUSED  a resident launch that the device refuses: not a failure
+ *              either, the steps go one per launch. */
 #define LBMFVM_FAULT_END 1
 #define LBMFVM_FAULT_POST 2
 #define LBMFVM_FAULT_SUBPOST 3
 #define LBMFVM_FAULT_LATE 4
+#define LBMFVM_FAULT_REFUSED 5
 int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind);
 
 /* Number of time steps taken since the last set_state. */

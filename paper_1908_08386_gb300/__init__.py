@@ -45,7 +45,8 @@ LBMFVM_FV_CENTRAL, LBMFVM_FV_QUICK = 0, 1
 FV_SCHEMES = {"central": LBMFVM_FV_CENTRAL, "quick": LBMFVM_FV_QUICK}
 LBMFVM_FV_SUBSTEPS_AUTO = 0
 # Test hooks of the bounded waits (lbmfvm_inject_fault)
-LBMFVM_FAULT_END, LBMFVM_FAULT_POST, LBMFVM_FAULT_SUBPOST, LBMFVM_FAULT_LATE = 1, 2, 3, 4
+LBMFVM_FAULT_END, LBMFVM_FAULT_POST, LBMFVM_FAULT_SUBPOST = 1, 2, 3
+LBMFVM_FAULT_LATE, LBMFVM_FAULT_REFUSED = 4, 5
 # Energy solvers
 LBMFVM_ENERGY_FV, LBMFVM_ENERGY_LBM_D2Q5 = 0, 1
 ENERGY = {"fv": LBMFVM_ENERGY_FV, "lbm": LBMFVM_ENERGY_LBM_D2Q5}

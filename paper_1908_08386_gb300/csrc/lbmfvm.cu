@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstddef>
@@ -340,6 +341,13 @@ struct lbmfvm {
     int res_shape, res_tiles;        // shape of resident launches (-1: none fits the active tiles) and its tiles
     bool res_general;                // they take the general energy update (QUICK or sub-steps)
     uint32_t res_seq;                // exchanges made since the resident tile list was built
+    int device;
+    unsigned long long user_id;      // of the caller's stream, unique in the process (0: unknown)
+    cudaEvent_t ev_res;              // end of the handle's last resident launch
+    int res_flight;                  // SMs its launches in flight hold at most
+    // places in the process-wide order of launches and joins (g_order): the last
+    // resident launch, the last join before and after a call's work
+    std::atomic<uint64_t> at_launch, at_in, at_out;
     uint32_t code_crc; // CRC-32 of the node codes, identifies the geometry in checkpoints
     int tile_w, tile_h;
     int tile_bw;      // columns between the tiles' rounding borders (TmaTile::BW)
@@ -597,7 +605,10 @@ void launch_one(const lbmfvm_t *h, int cur, cudaStream_t s, int stall = 0, bool 
     }
 }
 
+std::atomic<uint64_t> g_order{0};
+
 int join_in(lbmfvm_t *h) {
+    h->at_in = ++g_order;
     CU(h, cudaEventRecord(h->ev_in, h->user));
     CU(h, cudaStreamWaitEvent(h->s, h->ev_in, 0));
     return LBMFVM_OK;
@@ -606,6 +617,7 @@ int join_in(lbmfvm_t *h) {
 int join_out(lbmfvm_t *h) {
     CU(h, cudaEventRecord(h->ev_out, h->s));
     CU(h, cudaStreamWaitEvent(h->user, h->ev_out, 0));
+    h->at_out = ++g_order;
     return LBMFVM_OK;
 }
 
@@ -1458,6 +1470,12 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
         lbmfvm_destroy(h);
         return code;
     };
+    // (the per-thread default stream is another one in every thread)
+    if (cudaGetDevice(&h->device) != cudaSuccess || h->user == cudaStreamPerThread ||
+        cudaStreamGetId(h->user, &h->user_id) != cudaSuccess) {
+        h->user_id = 0;
+        cudaGetLastError();
+    }
     cudaError_t e = cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         h->s = nullptr;
@@ -1465,7 +1483,8 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
         return bail(LBMFVM_ERR_CUDA);
     }
     if (cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_res, cudaEventDisableTiming) != cudaSuccess) {
         fail(h, LBMFVM_ERR_CUDA, "cudaEventCreate failed");
         return bail(LBMFVM_ERR_CUDA);
     }
@@ -1537,15 +1556,62 @@ int fields_impl(lbmfvm_t *h, O *rho, O *u, O *v, O *T) {
 }  // namespace
 
 namespace {
-// Resident launches of one device go one after another: the blocks of two of
-// them that each got part of the SMs would wait for their missing ones.  The
-// last launch's event orders the next one, whichever handle, stream or thread
-// it comes from.
+// Handles with resident launches that may still be in flight (never destroyed:
+// handles may be, after the library's static objects).
 struct ResidentGate {
     std::mutex mu;
-    cudaEvent_t last[64] = {};
+    std::vector<lbmfvm_t *> flying;
 };
-ResidentGate g_resident;
+ResidentGate &g_resident = *new ResidentGate;
+
+// While it lives, this thread's calls neither break nor are refused by another
+// thread's stream capture (an event query counts as unsafe beside one).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Whether every launch in flight of o ends before what h queues now begins: they
+// share the caller's stream, and o's call had joined it before h's did.
+bool ordered_after(const lbmfvm_t *h, const lbmfvm_t *o) {
+    return h->user_id && o->user_id == h->user_id && o->at_out > o->at_launch && o->at_out < h->at_in;
+}
+
+// Whether a resident launch of h fits the SMs beside those that may run with
+// it (g_resident.mu held).  The blocks of two launches that each got part of
+// their SMs would wait for their missing ones, so the blocks in flight are at
+// most as many as the SMs: each then finds one that holds none of them.  A
+// launch that does not fit is not queued behind the others: that would make its
+// caller wait for whatever work another stream has before them.  Its steps go
+// one per launch, beside the resident ones.
+// Us per cavity step of N handles on streams of their own, all in one queue / this
+// rule / one launch per step: 64^2 FP32 N = 2 1.74 / 0.90 / 1.97, N = 32 1.75 /
+// 0.49 / 0.58; 300^2 FP32 3.13 / 3.13 / 2.69 and 3.09 / 2.20 / 2.25; 64^2
+// double-single 3.42 / 2.98 / 3.10 and 3.43 / 0.82 / 0.80; 64^2 FP64 5.1 / 8.7 /
+// 9.0 and 5.1 / 2.30 / 2.23 (on one stream they go one after another: 5.1).
+bool resident_room(lbmfvm_t *h) {
+    RelaxedCapture relaxed;
+    int used = 0;
+    auto &f = g_resident.flying;
+    for (size_t i = 0; i < f.size();) {
+        lbmfvm_t *o = f[i];
+        if (o->device != h->device) {
+            i++;
+            continue;
+        }
+        const cudaError_t e = cudaEventQuery(o->ev_res);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e != cudaErrorNotReady) {
+            o->res_flight = 0;
+            f.erase(f.begin() + i);
+            continue;
+        }
+        if (o != h && !ordered_after(h, o)) used += o->res_flight;
+        i++;
+    }
+    return used + h->res_tiles <= std::min(kResidentSlots, h->num_sms);
+}
 
 // Whether n steps from now may go into resident launches: enough of them to
 // pay for the launch (loading and storing the state), nothing injected, and
@@ -1557,9 +1623,12 @@ bool resident_steps(lbmfvm_t *h, int64_t n) {
 }
 
 // n steps in one resident launch (both population buffers and temperature
-// planes hold the state's two last steps only after one more ordinary step).
+// planes hold the state's two last steps only after one more ordinary step);
+// taken: whether there was room for it and the device accepted it.
 template <class S>
-int launch_resident(lbmfvm_t *h, int n) {
+int launch_resident(lbmfvm_t *h, int n, bool &taken) {
+    std::lock_guard<std::mutex> lock(g_resident.mu);
+    if (!resident_room(h)) return LBMFVM_OK;
     ResArgs<S> r{};
     r.a = args_for<S>(h, h->parity);
     r.fflags = h->base + h->L.fflags;
@@ -1586,16 +1655,22 @@ int launch_resident(lbmfvm_t *h, int n) {
             r.wait_ns = kWaitLimitNs / 50;
             break;
     }
+    const bool refused = h->fault_next == LBMFVM_FAULT_REFUSED;
     h->fault_next = 0;
-    int dev = 0;
-    CU(h, cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(h, LBMFVM_ERR_CUDA, "device %d", dev);
-    std::lock_guard<std::mutex> lock(g_resident.mu);
-    cudaEvent_t &last = g_resident.last[dev];
-    if (!last) CU(h, cudaEventCreateWithFlags(&last, cudaEventDisableTiming));
-    else CU(h, cudaStreamWaitEvent(h->s, last, 0));
-    CU(h, lbmfvm_fv::resident_launch<S>(h->res_shape, h->res_general, r, h->res_tiles, h->s));
-    CU(h, cudaEventRecord(last, h->s));
+    const cudaError_t e = refused ? cudaErrorCooperativeLaunchTooLarge
+                                  : lbmfvm_fv::resident_launch<S>(h->res_shape, h->res_general, r, h->res_tiles, h->s);
+    if (e != cudaSuccess) {
+        // the device has no room for the blocks at once (a share of its SMs): ordinary steps from now on
+        cudaGetLastError();
+        h->res_shape = -1;
+        return LBMFVM_OK;
+    }
+    taken = true;
+    h->at_launch = ++g_order;
+    auto &f = g_resident.flying;
+    if (std::find(f.begin(), f.end(), h) == f.end()) f.push_back(h);
+    h->res_flight = std::max(h->res_flight, h->res_tiles);
+    CU(h, cudaEventRecord(h->ev_res, h->s));
     h->res_seq += (uint32_t)n;
     h->parity ^= 1;
     h->steps += n;
@@ -1603,13 +1678,13 @@ int launch_resident(lbmfvm_t *h, int n) {
     return LBMFVM_OK;
 }
 
-int run_resident(lbmfvm_t *h, int n) {
+int run_resident(lbmfvm_t *h, int n, bool &taken) {
     switch (h->prec) {
-        case LBMFVM_F64: return launch_resident<double>(h, n);
-        case LBMFVM_F32: return launch_resident<float>(h, n);
-        case LBMFVM_F16: return launch_resident<__half>(h, n);
-        case LBMFVM_BF16: return launch_resident<__nv_bfloat16>(h, n);
-        case LBMFVM_F32X2: return launch_resident<dsf>(h, n);
+        case LBMFVM_F64: return launch_resident<double>(h, n, taken);
+        case LBMFVM_F32: return launch_resident<float>(h, n, taken);
+        case LBMFVM_F16: return launch_resident<__half>(h, n, taken);
+        case LBMFVM_BF16: return launch_resident<__nv_bfloat16>(h, n, taken);
+        case LBMFVM_F32X2: return launch_resident<dsf>(h, n, taken);
     }
     return LBMFVM_OK;
 }
@@ -1621,7 +1696,9 @@ int step_impl(lbmfvm_t *h, int64_t n) {
         while (n > 1) {
             int k = (int)std::min<int64_t>(n - 1, kResidentSteps);
             if (h->fault_next == LBMFVM_FAULT_SUBPOST) k = 1;
-            if (int r = run_resident(h, k)) return r;
+            bool taken = false;
+            if (int r = run_resident(h, k, taken)) return r;
+            if (!taken) break;
             n -= k;
         }
     }
@@ -1763,6 +1840,7 @@ int lbmfvm_inject_fault(lbmfvm_t *h, int32_t kind) {
             [[fallthrough]];
         case LBMFVM_FAULT_POST:
         case LBMFVM_FAULT_LATE:
+        case LBMFVM_FAULT_REFUSED:
             if (h->res_shape < 0 || h->res_tiles < 2)
                 return fail(h, LBMFVM_ERR_ARG, "the handle has no resident launches with an exchange");
             h->fault_next = kind;
@@ -1902,11 +1980,17 @@ int lbmfvm_params(const lbmfvm_t *h, double *nu, double *alpha, double *gbeta, d
 void lbmfvm_destroy(lbmfvm_t *h) {
     if (!h) return;
     if (h->s) cudaStreamSynchronize(h->s);
+    {
+        std::lock_guard<std::mutex> lock(g_resident.mu);
+        auto &f = g_resident.flying;
+        f.erase(std::remove(f.begin(), f.end(), h), f.end());
+    }
     if (h->graph) cudaGraphExecDestroy(h->graph);
     if (h->owns && h->base) cudaFree(h->base);
     if (h->host) cudaFreeHost(h->host);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->ev_out) cudaEventDestroy(h->ev_out);
+    if (h->ev_res) cudaEventDestroy(h->ev_res);
     if (h->s) cudaStreamDestroy(h->s);
     delete h;
 }

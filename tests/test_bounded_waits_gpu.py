@@ -89,6 +89,22 @@ def test_a_block_that_starts_late_is_waited_for(nx, ny, store, m):
     ref.close()
 
 
+@pytest.mark.parametrize("store,m", [("f32", 1), ("f64", 2)])
+def test_a_refused_resident_launch_leaves_ordinary_steps(store, m):
+    kw = dict(KW, alpha=0.05 * m, store=store, fv_substeps=m)
+    c, ref = L.Cavity(70, 90, **kw), L.Cavity(70, 90, kernel="tma", **kw)
+    for h in (c, ref):
+        h.set_state(*state(70, 90, 9))
+    L.lbmfvm_inject_fault(c.h, L.LBMFVM_FAULT_REFUSED)
+    for n in (60, 9):
+        c.step(n)
+        ref.step(n)
+    assert c.steps == ref.steps == 69
+    assert np.array_equal(np.stack(c.fields()), np.stack(ref.fields()))
+    c.close()
+    ref.close()
+
+
 def test_hooks_of_kernels_that_are_not_in_use_are_refused():
     for kw in (dict(tma_config=4, kernel="tma"), dict(store="f64"), dict(kernel="generic")):
         c = L.Cavity(40, 40, **dict(KW, **kw))
