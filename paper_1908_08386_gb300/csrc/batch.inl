@@ -238,8 +238,8 @@ int bcheck_h(lbmfvm_batch_t *b, lbmfvm_t *h, int code) {
 // than the GPU has SMs is bound by the latency of one tile rather than by
 // throughput: it takes the small-grid shape a single cavity of that size
 // would (64 x 8 for 32- and 16-bit storage, 32 x 8 with ring warps for
-// 64-bit), and its own shape again when the active set grows.  Shapes never
-// change results.
+// 64-bit), and its own shape again when the active set grows.  Shapes
+// change results by rounding at most (see the autotuner).
 int reshape_level(lbmfvm_batch_t *b, int l) {
     lbmfvm_t *h = b->lv[l];
     if (!b->auto_shape || !h || !h->use_tma || h->fv_quick || h->L.split || h->grid2) return LBMFVM_OK;

@@ -339,7 +339,7 @@ struct lbmfvm {
     uint64_t tiles_gen, graph_gen;   // tile-list generation, and the one the graph was captured with
     bool res_allowed;                // kernel and tile shape are the library's choice
     int res_shape, res_tiles;        // shape of resident launches (-1: none fits the active tiles) and its tiles
-    bool res_general;                // they take the general energy update (QUICK or sub-steps)
+    ResForm res_form;                // their kernel: general energy update (QUICK or sub-steps), tile borders beside walls
     uint32_t res_seq;                // exchanges made since the resident tile list was built
     int device;
     unsigned long long user_id;      // of the caller's stream, unique in the process (0: unknown)
@@ -952,13 +952,13 @@ TileHeader tile_header(const CavityDesc &cd, int c, int x0, int y0) {
 }
 
 // Blocks per SM of resident shape i for the handle's storage.
-cudaError_t res_prepare(const lbmfvm_t *h, int i, bool general, int *blocks) {
+cudaError_t res_prepare(const lbmfvm_t *h, int i, ResForm form, int *blocks) {
     switch (h->prec) {
-        case LBMFVM_F64: return lbmfvm_fv::resident_prepare<double>(i, general, blocks);
-        case LBMFVM_F16: return lbmfvm_fv::resident_prepare<__half>(i, general, blocks);
-        case LBMFVM_BF16: return lbmfvm_fv::resident_prepare<__nv_bfloat16>(i, general, blocks);
-        case LBMFVM_F32X2: return lbmfvm_fv::resident_prepare<dsf>(i, general, blocks);
-        default: return lbmfvm_fv::resident_prepare<float>(i, general, blocks);
+        case LBMFVM_F64: return lbmfvm_fv::resident_prepare<double>(i, form, blocks);
+        case LBMFVM_F16: return lbmfvm_fv::resident_prepare<__half>(i, form, blocks);
+        case LBMFVM_BF16: return lbmfvm_fv::resident_prepare<__nv_bfloat16>(i, form, blocks);
+        case LBMFVM_F32X2: return lbmfvm_fv::resident_prepare<dsf>(i, form, blocks);
+        default: return lbmfvm_fv::resident_prepare<float>(i, form, blocks);
     }
 }
 
@@ -971,9 +971,13 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
     if (!h->res_allowed || !h->L.mail_bytes || h->grid2) return LBMFVM_OK;
     const int slots = std::min(kResidentSlots, h->num_sms);
     auto active = [&](size_t c) { return h->atlas_cavs.empty() || h->atlas_active[c]; };
-    h->res_general = h->fv_quick;
+    // Row borders of the step kernel's tiles matter beside the north wall, and
+    // beside vertical walls whose nodes balance energy (a batch's may be any).
+    h->res_form = ResForm{h->fv_quick, !h->atlas_cavs.empty() || h->grid.bc[LBMFVM_SIDE_W] != LBMFVM_BC_DIRICHLET ||
+                                           h->grid.bc[LBMFVM_SIDE_E] != LBMFVM_BC_DIRICHLET ||
+                                           (h->grid.ny - 1) % h->tile_h == 0};
     for (size_t c = 0; c < table.size(); c++)
-        if (active(c) && table[c].substeps > 1) h->res_general = true;
+        if (active(c) && table[c].substeps > 1) h->res_form.general = true;
     std::vector<TileHeader> list;
     for (int i = 0; i < kResShapes; i++) {
         const lbmfvm_fv::ResShape sh = res_shape(h->prec, i);
@@ -983,7 +987,7 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
             if (active(c)) tiles += res_tiles_of(sh, table[c].nx, table[c].ny);
         if (tiles < 1 || tiles > slots || (size_t)tiles * sh.mail_bytes > h->L.mail_bytes) continue;
         int blocks = 0;
-        CU(h, res_prepare(h, i, h->res_general, &blocks));
+        CU(h, res_prepare(h, i, h->res_form, &blocks));
         if (blocks < 1) continue;
         for (size_t c = 0; c < table.size(); c++) {
             if (!active(c)) continue;
@@ -1203,7 +1207,9 @@ int check_device_status(lbmfvm_t *h) {
 // The fastest shape is kept and remembered for the storage precision and the
 // size class (the power of two of the nodes the tiles cover), so a class is
 // measured once per process.  Every shape computes the same arithmetic per
-// node, so the choice never changes results.  The population and temperature
+// node; in FP32 arithmetic a wall node's velocity as seen across a tile border is
+// the wall's own, which differs by rounding from the extrapolated one, so shapes
+// whose borders lie beside other walls differ by that rounding.  The population and temperature
 // buffers are cleared again afterwards.  Runs at creation, outside any stream
 // capture of the caller.
 constexpr int kTuneSteps = 32;
@@ -1658,7 +1664,7 @@ int launch_resident(lbmfvm_t *h, int n, bool &taken) {
     const bool refused = h->fault_next == LBMFVM_FAULT_REFUSED;
     h->fault_next = 0;
     const cudaError_t e = refused ? cudaErrorCooperativeLaunchTooLarge
-                                  : lbmfvm_fv::resident_launch<S>(h->res_shape, h->res_general, r, h->res_tiles, h->s);
+                                  : lbmfvm_fv::resident_launch<S>(h->res_shape, h->res_form, r, h->res_tiles, h->s);
     if (e != cudaSuccess) {
         // the device has no room for the blocks at once (a share of its SMs): ordinary steps from now on
         cudaGetLastError();

@@ -285,8 +285,24 @@ struct ResArgs {
 };
 
 // GENERAL: QUICK face values and energy sub-steps; else the central update,
-// one per step.
-template <class S, class G, bool GENERAL>
+// one per step.  BORDERS: a tile may hold a row border of the step kernel's tiles
+// beside a wall (bits 23 and 24 of info below).  FP32 arithmetic in tiles of more
+// than 8 rows (64-bit types round the two wall velocities alike; the step
+// kernel's tiles have 8 rows or more).  Us per step without / with it: 256^2 in
+// 32 x 16 2.21 / 2.23, 384^2 in 32 x 32 3.15 / 3.15, 512^2 in 64 x 32 5.55 / 5.8,
+// 512 x 384 with two sub-steps 8.07 / 8.5: a form of its own in the last shapes.
+template <class S, class G>
+constexpr bool res_borders() {
+    return std::is_same<typename Compute<S>::type, float>::value && G::TH > 8;
+}
+template <class S, class G>
+constexpr bool res_borders_apart() {
+    return res_borders<S, G>() && G::NPT > 2;
+}
+struct ResForm {
+    bool general, borders;
+};
+template <class S, class G, bool GENERAL, bool BORDERS>
 __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> r) {
     using C = typename Compute<S>::type;
     constexpr int TW = G::TW, TH = G::TH, FW = G::FW, PL = G::PL, RW = G::RW, NPT = G::NPT, BLOCK = G::BLOCK;
@@ -360,7 +376,11 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
     auto own_node = [&](int j) { return G::QUAD ? tid >> 2 : tid + j * G::NT; };
     const int lane4 = tid & 3;
 
-    // Own nodes: code, face flags, far-face flags (QUICK), wall side.
+    // Own nodes: code, face flags, far-face flags (QUICK), wall side; bits 23 and
+    // 24: the node above (below) is a wall node across a border of the step
+    // kernel's tiles inside this one, see the ring nodes below.  (The step kernel's
+    // borders between columns are borders of these tiles too, and the two nodes
+    // of a face between wall nodes lie on one side.)
     const bool computes = tid < G::NT;
     uint32_t info[NPT];
     constexpr uint32_t kDead = CODE_OUTSIDE;
@@ -380,6 +400,13 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                 if ((ff & FF_OPEN_S) && (r.fflags[k - pitch] & FF_OPEN_S)) far |= FF_OPEN_S;
             }
             info[j] = c | ((uint32_t)ff << 8) | (far << 16) | ((uint32_t)side_of(lx, ly, c) << 20);
+            if (BORDERS && m == 1) {
+                const int y = oy + ly;
+                if (ly + 1 < TH && (ff & FF_OPEN_N) && (y + 1) % r.tile_h == 0 && (decode(r.a.code[k + pitch]) & 3) == KIND_WALL)
+                    info[j] |= 1u << 23;
+                if (ly > 0 && (ff & FF_OPEN_S) && y % r.tile_h == 0 && (decode(r.a.code[k - pitch]) & 3) == KIND_WALL)
+                    info[j] |= 1u << 24;
+            }
             if ((c & 3) == KIND_SOLID) {
                 // inert nodes never change: their results are written once
 #pragma unroll
@@ -627,7 +654,21 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
                         const C ex = ((ff & FF_IN_W) ? C(0.5) : C(0)) + ((ff & FF_IN_E) ? C(0.5) : C(0));
                         const C ey = ((ff & FF_IN_S) ? C(0.5) : C(0)) + ((ff & FF_IN_N) ? C(0.5) : C(0));
                         const C TE = Tc[t + 1], TWt = Tc[t - 1], TN = Tc[t + FW], TS = Tc[t - FW];
-                        const C uE = RU[rr + 1], uW = RU[rr - 1], vN = RV[rr + RW], vS = RV[rr - RW];
+                        const C uE = RU[rr + 1], uW = RU[rr - 1];
+                        C vN, vS;
+                        if constexpr (BORDERS && NPT <= 2) {
+                            const C *wv = wall + 2 * ((c >> 20) & 7) + 1;
+                            vN = *(c >> 23 & 1u ? wv : RV + rr + RW);
+                            vS = *(c >> 24 & 1u ? wv : RV + rr - RW);
+                        } else {
+                            vN = RV[rr + RW];
+                            vS = RV[rr - RW];
+                            if (BORDERS && (c >> 23 & 3u)) {  // (two addresses more per node would spill)
+                                const C wv = wall[2 * ((c >> 20) & 7) + 1];
+                                if (c >> 23 & 1u) vN = wv;
+                                if (c >> 24 & 1u) vS = wv;
+                            }
+                        }
                         const bool oE = ff & FF_OPEN_E, oN = ff & FF_OPEN_N, oW = ff & FF_OPEN_W, oS = ff & FF_OPEN_S;
                         if (!GENERAL || (!r.quick && m == 1)) {
                             t1 = fv_update<C>(TP, uu[j], vv[j], ex, ey, alpha, oE, TE, uE, oN, TN, vN, oW, TWt, uW, oS,
@@ -759,9 +800,10 @@ template <class S>
 ResShape resident_shape(int i);
 // Blocks of the shape's kernel that fit an SM (its shared-memory limit set).
 template <class S>
-cudaError_t resident_prepare(int i, bool general, int *blocks_per_sm);
+cudaError_t resident_prepare(int i, lbmfvm_dev::ResForm form, int *blocks_per_sm);
 // Cooperative launch over `tiles` blocks.
 template <class S>
-cudaError_t resident_launch(int i, bool general, const lbmfvm_dev::ResArgs<S> &r, int tiles, cudaStream_t stream);
+cudaError_t resident_launch(int i, lbmfvm_dev::ResForm form, const lbmfvm_dev::ResArgs<S> &r, int tiles,
+                            cudaStream_t stream);
 
 }  // namespace lbmfvm_fv

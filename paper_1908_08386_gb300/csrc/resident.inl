@@ -12,26 +12,31 @@ using namespace lbmfvm_dev;
 namespace {
 
 template <class S, int I>
-const void *kernel_of(bool general) {
+const void *kernel_of(ResForm f) {
     using G = typename ResConfig<S, I>::G;
-    return general ? reinterpret_cast<const void *>(resident_kernel<S, G, true>)
-                   : reinterpret_cast<const void *>(resident_kernel<S, G, false>);
+    constexpr bool B = res_borders<S, G>();
+    if constexpr (res_borders_apart<S, G>())
+        if (!f.borders)
+            return f.general ? reinterpret_cast<const void *>(resident_kernel<S, G, true, false>)
+                             : reinterpret_cast<const void *>(resident_kernel<S, G, false, false>);
+    return f.general ? reinterpret_cast<const void *>(resident_kernel<S, G, true, B>)
+                     : reinterpret_cast<const void *>(resident_kernel<S, G, false, B>);
 }
 
 template <class S, int I>
-cudaError_t prepare_i(bool general, int *blocks) {
+cudaError_t prepare_i(ResForm form, int *blocks) {
     using G = typename ResConfig<S, I>::G;
-    const void *k = kernel_of<S, I>(general);
+    const void *k = kernel_of<S, I>(form);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, G::BLOCK, G::SMEM);
     return e;
 }
 
 template <class S, int I>
-cudaError_t launch_i(bool general, const ResArgs<S> &r, int tiles, cudaStream_t stream) {
+cudaError_t launch_i(ResForm form, const ResArgs<S> &r, int tiles, cudaStream_t stream) {
     using G = typename ResConfig<S, I>::G;
     void *args[] = {const_cast<ResArgs<S> *>(&r)};
-    return cudaLaunchCooperativeKernel(kernel_of<S, I>(general), dim3(tiles), dim3(G::BLOCK), args, G::SMEM, stream);
+    return cudaLaunchCooperativeKernel(kernel_of<S, I>(form), dim3(tiles), dim3(G::BLOCK), args, G::SMEM, stream);
 }
 
 template <class S, int I>
@@ -61,15 +66,15 @@ ResShape resident_shape(int i) {
     return ResShape{};
 }
 template <class S>
-cudaError_t resident_prepare(int i, bool general, int *blocks) {
-#define CALL(I) (prepare_i<S, I>(general, blocks))
+cudaError_t resident_prepare(int i, ResForm form, int *blocks) {
+#define CALL(I) (prepare_i<S, I>(form, blocks))
     LBMFVM_RES_SWITCH(i, CALL)
 #undef CALL
     return cudaErrorInvalidValue;
 }
 template <class S>
-cudaError_t resident_launch(int i, bool general, const ResArgs<S> &r, int tiles, cudaStream_t stream) {
-#define CALL(I) (launch_i<S, I>(general, r, tiles, stream))
+cudaError_t resident_launch(int i, ResForm form, const ResArgs<S> &r, int tiles, cudaStream_t stream) {
+#define CALL(I) (launch_i<S, I>(form, r, tiles, stream))
     LBMFVM_RES_SWITCH(i, CALL)
 #undef CALL
     return cudaErrorInvalidValue;
@@ -77,7 +82,7 @@ cudaError_t resident_launch(int i, bool general, const ResArgs<S> &r, int tiles,
 
 #define LBMFVM_RESIDENT_INSTANTIATE(S)                                       \
     template ResShape resident_shape<S>(int);                                \
-    template cudaError_t resident_prepare<S>(int, bool, int *);              \
-    template cudaError_t resident_launch<S>(int, bool, const ResArgs<S> &, int, cudaStream_t);
+    template cudaError_t resident_prepare<S>(int, ResForm, int *);              \
+    template cudaError_t resident_launch<S>(int, ResForm, const ResArgs<S> &, int, cudaStream_t);
 
 }  // namespace lbmfvm_fv
