@@ -1034,8 +1034,8 @@ constexpr int kTmaConfigFv = 1;
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per wait
 constexpr int kErrTimeout = 1;
 // Test hooks of the step kernel, block 0: its first staged load is never issued;
-// its first warp takes the end mark of the block's tiles (copying-warp shape) for
-// a wait that ran out.
+// its first warp, at the end mark of the block's tiles (copying-warp shape), does
+// what it does when a wait runs out.
 constexpr int kStallLoad = 1, kStallEnd = 2;
 
 namespace tma {
@@ -1260,20 +1260,19 @@ __global__ void __launch_bounds__(G::BLOCK, G::MINB)
 
     for (int k = 0; G::PW || k < *known; k++) {
         unsigned char *stg = stage(k);
-        bool landed = tma::mbar_wait_bounded(&bars[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u, kWaitLimitNs);
-        bool end = false;
-        if constexpr (G::PW) {
-            end = landed && !valid[k % G::STAGES];
-            if (end && a.stall == kStallEnd && blockIdx.x == 0 && tid < 32) landed = end = false;
-        }
+        const bool landed = tma::mbar_wait_bounded(&bars[k % G::STAGES], (uint32_t)(k / G::STAGES) & 1u, kWaitLimitNs);
         if (!landed) {
             atomicOr(abort_flag, 1);
             atomicOr(a.err, kErrTimeout);
         }
         if constexpr (G::PW) {
-            if (end) {
-                // a thread whose wait ran out as the mark came does not know of
-                // the end and goes on to this tile's barrier: meet it there
+            if (landed && !valid[k % G::STAGES]) {
+                // The end mark.  A thread whose wait ran out as it came does not
+                // know of the end and goes on to this tile's barrier: meet it there.
+                if (a.stall == kStallEnd && blockIdx.x == 0 && tid < 32) {
+                    atomicOr(abort_flag, 1);
+                    atomicOr(a.err, kErrTimeout);
+                }
                 asm volatile("bar.sync 1, %0;" ::"n"(G::CONSUMERS) : "memory");
                 break;
             }
