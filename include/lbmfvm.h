@@ -81,14 +81,15 @@ extern "C" {
  *            boundary, every storage type).
  * AUTO takes TMA where it applies and GENERIC otherwise; with a tile shape left
  * to the library too (tma_config TMA_DEFAULT or TMA_AUTOTUNE), grids and batches
- * whose tiles fit the SMs one per block (up to about 300,000 nodes in FP32, 75,000
- * in 64-bit types) run all but the last of eight or more steps of a call in one
+ * whose tiles fit the SMs one per block (up to about 150,000 nodes in FP32 and 16-bit
+ * storage, 300,000 where the larger tiles pay, 75,000 in 64-bit types) run all but
+ * the last of eight or more steps of a call (24 or more in the larger tiles) in one
  * launch that keeps the state on the chip, with the same results.  The blocks of
  * such a launch wait for one another: other work that keeps some of them off
  * their SMs for more than two minutes makes the call fail with
- * LBMFVM_ERR_TIMEOUT.  A call
- * takes its steps one per launch where the device has no room for such a launch
- * beside those of handles on other streams that are still in flight, and while the
+ * LBMFVM_ERR_TIMEOUT.  A call takes its steps one per launch where the device has no
+ * room for such a launch beside those of handles on other streams that are still
+ * in flight, and while the
  * stream is being captured. */
 #define LBMFVM_KERNEL_AUTO 0
 #define LBMFVM_KERNEL_GENERIC 1
@@ -184,8 +185,9 @@ typedef struct {
                                or 4 (64-bit), which spread it over more SMs;
                                otherwise 4 for 32-bit storage whose population
                                buffers and temperature planes fit in the L2, 5
-                               beyond it and for 16-bit storage, 3 for 64-bit: the
-                               fastest measured on 64^2 to 4096^2 cavities.
+                               beyond it and for 16-bit storage, 3 for 64-bit (on
+                               single sizes another shape can be a few percent
+                               faster).
                                LBMFVM_TMA_AUTOTUNE times every shape (a
                                captured graph of 32 launches, replayed twice)
                                on the handle's own grid at create and keeps

@@ -36,6 +36,10 @@ constexpr int kGraphSteps = 64;      // launches per captured graph (even)
 // state once (about 8 us with the launch) and saves 1.4 us or more a step
 // (9 steps of 64^2 FP32: 22.7 us against 39.4; of 512^2: 68.6 against 74.7).
 constexpr int kResidentMin = 8;
+// Their 64-column tiles load and store more of the state per SM and gain less a
+// step (see resident_pays): 576 x 512 FP32, 16 steps 6.51 us each against 6.65, 8
+// steps 7.5 against 6.7.
+constexpr int kResidentMinWide = 24;
 constexpr int kResidentSteps = 1 << 16;  // steps of one resident launch at most
 constexpr int kResidualBlocks = 608; // 4 x 152 SMs
 // Reduction scratch (doubles): kResidualSums partials per residual block,
@@ -339,6 +343,7 @@ struct lbmfvm {
     uint64_t tiles_gen, graph_gen;   // tile-list generation, and the one the graph was captured with
     bool res_allowed;                // kernel and tile shape are the library's choice
     int res_shape, res_tiles;        // shape of resident launches (-1: none fits the active tiles) and its tiles
+    int res_min;                     // steps from which they are worth it
     ResForm res_form;                // their kernel: general energy update (QUICK or sub-steps), tile borders beside walls
     uint32_t res_seq;                // exchanges made since the resident tile list was built
     int device;
@@ -962,6 +967,22 @@ cudaError_t res_prepare(const lbmfvm_t *h, int i, ResForm form, int *blocks) {
     }
 }
 
+// Whether many steps of one energy update each are faster in `tiles` resident
+// tiles of 64 columns than one per launch.  Those take as long however few of
+// the SMs they fill (FP32 64 x 32 5.6 us a step, with QUICK 7.0; 16-bit 64 x 32
+// 6.0, 64 x 40 7.3, with QUICK 7.4 and 10), while the step kernel's time grows with
+// the nodes.  Us per step resident / one launch per step, 256 steps: FP32 448^2 (98
+// tiles) 5.70 / 5.64, 398 x 556 (126) 5.8 / 6.1, 512^2 (128) 5.65 / 5.68, 640 x 480
+// (150) 5.71 / 6.31; with QUICK 448^2 6.99 / 7.37, 512^2 6.92 / 8.04; FP16 448^2
+// 6.0 / 5.2, 512^2 5.96 / 6.18, 640 x 560 (140 of 64 x 40) 7.18 / 6.72, 600^2 (150)
+// 7.19 / 8.20, 1216 x 320 (152) 7.23 / 6.79; with QUICK 600^2 10.0 / 10.0, 640 x 560
+// 9.9 / 8.8.  Sub-steps save three launches a step each and always pay (512 x 384,
+// two: 8.1 / 22).
+bool resident_pays(const lbmfvm_t *h, long long tiles, int slots) {
+    if (store_size(h->prec) == 2) return !h->fv_quick && tiles * 20 >= slots * 19;
+    return true;
+}
+
 // The resident launches' tile list: the smallest shape whose tiles over the
 // active cavities fit one per SM, if any.  A new list starts with cleared
 // mailboxes, so that no tag of an earlier list can be taken for one of its own.
@@ -976,8 +997,10 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
     h->res_form = ResForm{h->fv_quick, !h->atlas_cavs.empty() || h->grid.bc[LBMFVM_SIDE_W] != LBMFVM_BC_DIRICHLET ||
                                            h->grid.bc[LBMFVM_SIDE_E] != LBMFVM_BC_DIRICHLET ||
                                            (h->grid.ny - 1) % h->tile_h == 0};
+    bool substeps = false;
     for (size_t c = 0; c < table.size(); c++)
-        if (active(c) && table[c].substeps > 1) h->res_form.general = true;
+        if (active(c) && table[c].substeps > 1) substeps = true;
+    if (substeps) h->res_form.general = true;
     std::vector<TileHeader> list;
     for (int i = 0; i < kResShapes; i++) {
         const lbmfvm_fv::ResShape sh = res_shape(h->prec, i);
@@ -986,6 +1009,8 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
         for (size_t c = 0; c < table.size(); c++)
             if (active(c)) tiles += res_tiles_of(sh, table[c].nx, table[c].ny);
         if (tiles < 1 || tiles > slots || (size_t)tiles * sh.mail_bytes > h->L.mail_bytes) continue;
+        const bool wide = sh.TW >= 64 && !substeps;
+        if (wide && !resident_pays(h, tiles, slots)) continue;
         int blocks = 0;
         CU(h, res_prepare(h, i, h->res_form, &blocks));
         if (blocks < 1) continue;
@@ -998,6 +1023,7 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
         }
         h->res_shape = i;
         h->res_tiles = (int)tiles;
+        h->res_min = wide ? kResidentMinWide : kResidentMin;
         h->res_seq = 0;
         CU(h, cudaMemsetAsync(h->base + h->L.mail, 0, (size_t)tiles * sh.mail_bytes, h->s));
         CU(h, cudaMemcpyAsync(h->base + h->L.rtiles, list.data(), list.size() * sizeof(TileHeader),
@@ -1016,8 +1042,9 @@ int upload_resident(lbmfvm_t *h, const std::vector<CavityDesc> &table) {
 // rounds of them first), so that each block gets as many as the next and the
 // blocks that take one more tile in the last round have the fewest.  The order
 // of the tiles never changes results.  Us per step, row by row / spread (shape):
-// FP32 600^2 10.8 / 7.6 (4), 400 x 900 9.1 / 7.7 (4), 1024^2 16.0 / 16.3 (4), 4096^2
-// 209 / 206 (5); FP16 530^2 8.9 / 6.9, 1024^2 14.7 / 13.4, 4096^2 167 / 163 (5).
+// FP32 600^2 10.8 / 7.5 (4), 400 x 900 9.1 / 7.5 (4), 800^2 11.5 / 11.2 (4), 1024^2 16.0 /
+// 15.6 (4), 4096^2 212 / 208 (5); FP16 530^2 9.0 / 6.9, 1024^2 14.9 / 13.6, 4096^2 172 /
+// 168 (5).
 void spread_wall_tiles(std::vector<TileHeader> &list, int blocks, int tw, int th) {
     if (blocks < 1 || (int)list.size() <= blocks) return;
     std::vector<TileHeader> wall, rest;
@@ -1421,12 +1448,16 @@ int create_impl(const lbmfvm_grid_t *grid, const uint8_t *mask, double nu, doubl
     h->prec = opts.store;
     h->tile_y = opts.tile_y ? opts.tile_y : 8;
     h->use_tma = tma_ok && opts.kernel != LBMFVM_KERNEL_GENERIC;
-    // the default shapes are the fastest measured ones: two blocks of 32 x 16
-    // per SM with ring warps for 32-bit storage that fits the L2 (600^2: 7.6 us
-    // against 8.8, 900^2 12.7 against 13.7; 1024^2 16.3 against 15.6), 64 x 16 with
-    // a copying warp beyond it (4096^2: 206 against 215) and for 16-bit storage
-    // (1024^2: 13.4 against 14.4; 4096^2: 163 against 171), two blocks of 32 x 8
-    // per SM for 64-bit.  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
+    // the default shapes: two blocks of 32 x 16 per SM with ring warps for 32-bit
+    // storage that fits the L2, 64 x 16 with a copying warp beyond it and for
+    // 16-bit storage, two blocks of 32 x 8 per SM for 64-bit.  Of 41 FP32 sizes from
+    // 448^2 to 1344 x 1152 the first is faster at 29 (600^2 7.5 us against 8.9,
+    // 900^2 12.6 / 13.8, 1024 x 1100 16.7 / 17.7), within 1 % at 9 and slower at
+    // three (700^2 9.2 / 9.1, 1024^2 16.0 / 15.3, 1024 x 1040 16.3 / 15.6), 4 % on
+    // average; what decides is how the tiles divide over the blocks, with no size
+    // from which the other wins.  4096^2: 215 against 206.  Of 26 16-bit sizes the
+    // second is faster at 10 (1024^2 13.6 / 14.4, 960^2 12.2 / 13.1; 4096^2 163 / 171),
+    // slower at 10 (600^2 8.2 / 7.5, 900^2 12.5 / 12.1).  A grid with fewer 64 x 16 (64-bit: 32 x 8) tiles than
     // SMs is bound by the latency of one tile, not by the SMs' throughput, and
     // takes the smaller tiles that spread it over more SMs: 64 x 8 (two blocks
     // per SM) for 32- and 16-bit storage, 32 x 8 with ring warps for 64-bit.
@@ -1597,9 +1628,10 @@ bool ordered_after(const lbmfvm_t *h, const lbmfvm_t *o) {
 // double-single 3.42 / 2.98 / 3.10 and 3.43 / 0.82 / 0.80; 64^2 FP64 5.1 / 8.7 /
 // 9.0 and 5.1 / 2.30 / 2.23 (on one stream they go one after another: 5.1).
 bool resident_room(lbmfvm_t *h) {
+    auto &f = g_resident.flying;
+    if (f.empty() || (f.size() == 1 && f[0] == h)) return true;
     RelaxedCapture relaxed;
     int used = 0;
-    auto &f = g_resident.flying;
     for (size_t i = 0; i < f.size();) {
         lbmfvm_t *o = f[i];
         if (o->device != h->device) {
@@ -1623,7 +1655,7 @@ bool resident_room(lbmfvm_t *h) {
 // pay for the launch (loading and storing the state), nothing injected, and
 // no capture by the caller (tags count on, so a launch cannot be replayed).
 bool resident_steps(lbmfvm_t *h, int64_t n) {
-    if (h->res_shape < 0 || h->stall_next || n < kResidentMin) return false;
+    if (h->res_shape < 0 || h->stall_next || n < h->res_min) return false;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(h->s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }

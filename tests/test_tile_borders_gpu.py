@@ -22,7 +22,8 @@ def start(c, seed=3):
 
 # the last row (column) alone in a tile of 8 or 16 rows (64 columns), inside resident tiles of 16, 32 and 40 rows and at
 # their borders
-@pytest.mark.parametrize("nx,ny", [(100, 9), (65, 65), (256, 265), (257, 265), (321, 201), (300, 273), (503, 497), (610, 489)])
+@pytest.mark.parametrize("nx,ny", [(100, 9), (65, 65), (256, 265), (257, 265), (321, 201), (300, 273), (503, 497), (610, 489), (640, 465),
+                                   (600, 600)])
 @pytest.mark.parametrize("store", ["f32", "f16", "bf16"])
 @pytest.mark.parametrize("scheme,m,lid", [("central", 1, 0.0), ("central", 1, 0.05), ("quick", 1, 0.0), ("central", 2, 0.0)])
 def test_resident_steps_at_tile_borders_beside_walls(nx, ny, store, scheme, m, lid):
