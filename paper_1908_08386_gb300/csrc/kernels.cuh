@@ -127,11 +127,11 @@ __device__ __forceinline__ dsf operator*(dsf x, dsf y) {
 __device__ __forceinline__ dsf &operator+=(dsf &x, dsf y) { return x = x + y; }
 
 // Cheaper forms for sums of several terms (the double-single step is bound by
-// the number of its FP32 instructions: moments, energy balance and collision of
-// a node took about 1700, now 1180; a batch of 812,000 nodes 88 us a step, now
-// 62, and its deviation from FP64 fell with the longer reciprocal).  ds_add and ds_fma leave the low part
-// unnormalised (a few ulp of the high part): adding such values loses nothing
-// more, since the low parts are only summed; ds_norm renormalises once at the
+// the number of its FP32 instructions: a step of 512^2 took 1970 thread
+// instructions a node, now 1400; a batch of 812,000 nodes 88 us a step, now 62;
+// its fields' deviation from FP64 fell with the longer reciprocal).  ds_add and
+// ds_fma leave the low part unnormalised (a few ulp of the high part): adding
+// such values loses nothing more, since the low parts are only summed; ds_norm renormalises once at the
 // end of a chain, or before a value becomes a factor.  ds_mul_u takes
 // unnormalised factors (it keeps the product of the low parts).  An addition is
 // 8 instructions instead of 11, a fused a b + c 12 (15 normalised) instead of

@@ -6,11 +6,12 @@
 // the tile's border with its neighbours, so a step costs the tile's arithmetic
 // and one exchange through the L2 instead of a launch, a pipeline fill and a
 // drain, which bound small cavities whatever their size.  Measured (us per
-// step, one launch per step -> resident): FP32 64^2 3.68 -> 1.68, 128^2 3.98 ->
-// 1.89, 256^2 4.62 -> 2.16, 384^2 4.93 -> 3.19, 512^2 7.55 -> 5.89; FP16 256^2
-// 4.45 -> 2.28; double-single 64^2 5.82 -> 3.39, 128^2 5.76 -> 3.04, 192^2 5.95 ->
-// 3.57, 256^2 8.5 -> 6.3; FP64 64^2 21.0 -> 5.0, 128^2 21.0 -> 9.1, 192^2 21.1 ->
-// 15.6; 512 x 384 with QUICK and two sub-steps (four launches) 27.2 -> 10.3.
+// step, one launch per step -> resident, 64 or more steps): FP32 64^2 3.55 -> 1.70,
+// 128^2 3.86 -> 1.74, 256^2 4.52 -> 2.23, 384^2 4.81 -> 3.18, 512^2 5.7 -> 5.6; FP16
+// 256^2 4.40 -> 2.15; double-single 64^2 5.80 -> 3.46, 128^2 5.82 -> 3.07, 192^2 5.96
+// -> 3.62, 256^2 8.5 -> 6.1; FP64 64^2 17.2 -> 5.1, 128^2 17.3 -> 9.2, 192^2 17.4 ->
+// 15.7; 512 x 384 with two sub-steps (four launches) 22 -> 8.1, with QUICK and three
+// 32 -> 13.
 // What bounds it now: the exchange (about 1.1 us) and, for the 64-bit types,
 // the dependent chain of one node's operations.
 //
@@ -764,7 +765,9 @@ __global__ void __launch_bounds__(G::BLOCK, 1) resident_kernel(const ResArgs<S> 
 
 // Tile shapes, smallest first: the host takes the first one whose tiles fit
 // the SMs one per block.  Fewer nodes per SM mean a shorter step until the
-// exchange dominates, so the smallest shape that fits is the fastest.  Where
+// exchange dominates, so the smallest shape that fits is the fastest (the
+// 64-column ones not always faster than one launch per step, see the host's
+// resident_pays).  Where
 // no shape fits, or only one whose registers spill, one launch per step is the
 // faster (f32 64 x 40 tiles at 600^2: 9.2 us against 9.0; double-single 32 x 32
 // at 320^2: 32.5 against 15.7; FP64 74 against 63), so the lists end there.
